@@ -1169,6 +1169,15 @@ __global__ void k_restrict32(int n, const float* __restrict__ f, float* __restri
   c[split_index(I, J, K, nc)] = 0.125f * acc;
 }
 
+// 1/x within 1 ulp for a normal x, without the scaling of subnormal divisors
+// that __fdividef carries: num * rcp_approx(det) equals __fdividef(num, det)
+// for the determinants of the pointwise solve, which are >= 1.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Pointwise solve of the linearised 3x3 system (q frozen):
 //   [ 1   kap  0  ] [dp]   [r1 + tau/h^2 sum d_mu]
 //   [ -q  1    6g ] [dm] = [r2 + g sum d_om      ]
@@ -1181,12 +1190,54 @@ __device__ __forceinline__ void lin_point(const LvlF& L, float sp, float sm_, fl
   const float st3 = fmaf(L.gh, sp, r3);
   const float Q = q + L.Q0;
   const float det = fmaf(L.kap, Q, 1.0f);
-  // the division by the 2x2 determinant within 2 ulp (__fdividef): an FP32
-  // preconditioner step, and the IEEE division was a fifth of the sweep's
-  // instructions
-  dm = __fdividef(fmaf(Q, st1, fmaf(-L.g6, st3, st2)), det);
+  // the division by the 2x2 determinant within 2 ulp: an FP32 preconditioner
+  // step, and the IEEE division was a fifth of the sweep's instructions
+  dm = fmaf(Q, st1, fmaf(-L.g6, st3, st2)) * rcp_approx(det);
   dp = fmaf(-L.kap, dm, st1);
   dw = fmaf(-L.g3, dp, st3);
+}
+
+// Two cells at once: sm_103a adds and multiplies two FP32 values in one
+// instruction (add / fma .f32x2), each rounded as the scalar one.
+__device__ __forceinline__ unsigned long long f2_bits(float2 a) {
+  return *reinterpret_cast<unsigned long long*>(&a);
+}
+__device__ __forceinline__ float2 f2_of(unsigned long long u) {
+  return *reinterpret_cast<float2*>(&u);
+}
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+  return f2_of(r);
+}
+__device__ __forceinline__ float2 f2_all(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
+  return f2_fma(b, f2_all(-1.f), a);                 // a - b, one rounding
+}
+__device__ __forceinline__ float2 ldg2(const float* p) {
+  return __ldg(reinterpret_cast<const float2*>(p));
+}
+
+// lin_point on two cells.
+__device__ __forceinline__ void lin_point2(const LvlF& L, float2 sp, float2 sm_, float2 sw,
+                                           float2 q, float2 r1, float2 r2, float2 r3, float2& dp,
+                                           float2& dm, float2& dw) {
+  const float2 st1 = f2_fma(f2_all(L.tg), sm_, r1);
+  const float2 st2 = f2_fma(f2_all(L.g), sw, r2);
+  const float2 st3 = f2_fma(f2_all(L.gh), sp, r3);
+  const float2 Q = f2_add(q, f2_all(L.Q0));
+  const float2 det = f2_fma(f2_all(L.kap), Q, f2_all(1.0f));
+  const float2 num = f2_fma(Q, st1, f2_fma(f2_all(-L.g6), st3, st2));
+  dm = make_float2(num.x * rcp_approx(det.x), num.y * rcp_approx(det.y));
+  dp = f2_fma(f2_all(-L.kap), dm, st1);
+  dw = f2_fma(f2_all(-L.g3), dp, st3);
 }
 
 // One colour of a linear red-black sweep on split-layout fields: thread t
@@ -1220,68 +1271,139 @@ __global__ void k_lin_smooth32(LvlF L, int colour, float* d1, float* d2, float* 
   d3[s.c] = dw;
 }
 
-// The same colour pass with two adjacent cells of the colour's half-row per
-// thread (positions p0 = 2t and p0 + 1; n a multiple of 4, so every pair is
-// 8-byte aligned): own r, q, the y and z neighbours and the results move as
-// float2, and the pair's x neighbours in the other half are that half's
-// pair (p0, p0 + 1) plus one cell on the side the colour's offset sigma =
-// (j + k + colour) & 1 points to.  Same sums in the same order as above.
-template <bool ZERO>
-__global__ void k_lin_smooth32x2(LvlF L, int colour, float* d1, float* d2, float* d3,
-                                 const float* __restrict__ r1, const float* __restrict__ r2,
-                                 const float* __restrict__ r3, const float* __restrict__ q) {
+// ---------------------------------------------------------------------------
+// Smoothing passes that march in z (n a multiple of 4).  A thread owns two
+// adjacent positions of a half-row (float2 moves; two cells of one colour, or
+// of both) over `zc` planes and carries the other colour's values at its
+// positions from plane to plane: each value of d comes into the SM once per
+// column of planes (and once per row of the block in y, from L1) instead of
+// three times.  The passes of one plane per thread before moved 67 B a cell
+// between L2 and the SMs for the 40 B a Jacobi sweep needs, and ran at that
+// rate on the grids that L2 holds too.  One damped Jacobi sweep, in-graph, us,
+// before / now: 64^3 3.9 / 2.7, 96^3 7.5 / 5.9, 128^3 13.2 / 10.4, 256^3 125 /
+// 101 (98 % of the copy bandwidth), 42 x 64^3 85 / 68; one colour pass: 24^3
+// 2.1 / 1.6, 64^3 2.3 / 2.1, 128^3 6.6 / 5.4, 256^3 58 / 52.  Same sums in the
+// same order as the one-cell passes: bit-identical.
+// ---------------------------------------------------------------------------
+
+// Neighbour sums ((xm + xp) + (ym + yp)) + (zm + zp) of two adjacent cells of
+// one colour: o their positions' values of the other colour, e the third x
+// neighbour, above the pair where the row's offset sg = (j + k + colour) & 1 is
+// 1 and below it else.
+__device__ __forceinline__ float2 nbsum2(float2 o, float e, bool sg, float2 y0, float2 y1,
+                                         float2 z0, float2 z1) {
+  const float2 x = f2_add(o, sg ? make_float2(o.y, e) : make_float2(e, o.x));
+  return f2_add(f2_add(x, f2_add(y0, y1)), f2_add(z0, z1));
+}
+
+// A thread's place in a marching pass: its positions p, p + 1 of row j, planes
+// [k0, k1) of one ensemble member, and in-plane offsets (without the colour's
+// half-row) of its cells, the rows beside them and the x neighbours beyond.
+struct MarchCell {
+  size_t moff;
+  int k0, k1, j, c, ym, yp, xl, xr;
+  bool on;
+  __device__ __forceinline__ MarchCell(int n, int zc) {
+    const int half = n >> 1, p = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    int zb = blockIdx.z;
+    moff = (size_t)member_of(zb, (n + zc - 1) / zc) * n * n * n;
+    j = blockIdx.y * blockDim.y + threadIdx.y;
+    on = p < half && j < n;
+    k0 = zb * zc;
+    k1 = min(n, k0 + zc);
+    c = j * n + p;
+    ym = (j == 0 ? n - 1 : j - 1) * n + p;
+    yp = (j + 1 == n ? 0 : j + 1) * n + p;
+    xl = j * n + (p == 0 ? half - 1 : p - 1);
+    xr = j * n + (p + 2 >= half ? 0 : p + 2);
+  }
+};
+
+// Blocks of a marching pass: rows of at most 32 threads, 128 threads a block
+// (64 where the grid would not give every SM one of 128), and the most planes
+// a thread (4, 2 or 1) that leave 400 blocks: an SM holds four of them.
+struct March {
+  dim3 grid, block;
+  int zc;
+};
+inline March march(int n, int members) {
+  const int row = n / 4, parts = (row + 31) / 32, bx = (row + parts - 1) / parts;
+  const int64_t threads = (int64_t)row * n * n * members;
+  int by = (threads < 2 * 152 * 128 ? 64 : 128) / bx;
+  by = by < 1 ? 1 : by > n ? n : by;
+  March m;
+  m.block = dim3(bx, by, 1);
+  m.grid = dim3((row + bx - 1) / bx, (n + by - 1) / by, 1);
+  m.zc = 4;
+  while (m.zc > 1 && (int64_t)m.grid.x * m.grid.y * ((n + m.zc - 1) / m.zc) * members < 400)
+    m.zc >>= 1;
+  m.grid.z = (unsigned)((n + m.zc - 1) / m.zc * members);
+  return m;
+}
+
+// One colour of a linear red-black sweep.
+__global__ void __launch_bounds__(128, 6) k_lin_smooth32m(
+    LvlF L, int colour, int zc, float* d1, float* d2, float* d3, const float* __restrict__ r1,
+    const float* __restrict__ r2, const float* __restrict__ r3, const float* __restrict__ q) {
   pdl_wait();
   pdl_trigger();
-  const int n = L.n, half = n >> 1;
-  const int p0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  const int n = L.n, half = n >> 1, nn = n * n;
+  const MarchCell M(n, zc);
+  if (!M.on) return;
+  const int own = colour * half, oc = half - own;    // the colours' halves of a row
+  float* const d[3] = {d1 + M.moff, d2 + M.moff, d3 + M.moff};
+  const float* const rq[4] = {r1 + M.moff, r2 + M.moff, r3 + M.moff, q + M.moff};
+  float2 zm[3], zc_[3];
+  const size_t gm = (size_t)(M.k0 == 0 ? n - 1 : M.k0 - 1) * nn;
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    zm[f] = ldg2(d[f] + gm + oc + M.c);
+    zc_[f] = ldg2(d[f] + (size_t)M.k0 * nn + oc + M.c);
+  }
+#pragma unroll 1
+  for (int k = M.k0; k < M.k1; ++k) {
+    const size_t g = (size_t)k * nn, gp = (size_t)(k + 1 == n ? 0 : k + 1) * nn;
+    const bool sg = (M.j + k + colour) & 1;
+    float2 v[4], sum[3], zp[3], x[3];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) v[f] = ldg2(rq[f] + g + own + M.c);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      const float* const o = d[f] + g + oc;
+      zp[f] = ldg2(d[f] + gp + oc + M.c);
+      sum[f] = nbsum2(zc_[f], __ldg(o + (sg ? M.xr : M.xl)), sg, ldg2(o + M.ym), ldg2(o + M.yp),
+                      zm[f], zp[f]);
+    }
+    lin_point2(L, sum[0], sum[1], sum[2], v[3], v[0], v[1], v[2], x[0], x[1], x[2]);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      *reinterpret_cast<float2*>(d[f] + g + own + M.c) = x[f];
+      zm[f] = zc_[f];
+      zc_[f] = zp[f];
+    }
+  }
+}
+
+// The first colour-0 pass from d = 0 (n a multiple of 4): no neighbour is read.
+__global__ void k_lin_smooth32_zero(LvlF L, float* __restrict__ d1, float* __restrict__ d2,
+                                    float* __restrict__ d3, const float* __restrict__ r1,
+                                    const float* __restrict__ r2, const float* __restrict__ r3,
+                                    const float* __restrict__ q) {
+  pdl_wait();
+  pdl_trigger();
+  const int n = L.n;
+  const int p = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z;
   const size_t off = (size_t)member_of(k, n) * n * n * n;
-  if (p0 >= half || j >= n) return;
-  d1 += off, d2 += off, d3 += off, r1 += off, r2 += off, r3 += off, q += off;
-  const int sigma = (j + k + colour) & 1;
-  const int jm = (j == 0) ? n - 1 : j - 1, jp = (j + 1 == n) ? 0 : j + 1;
-  const int km = (k == 0) ? n - 1 : k - 1, kp = (k + 1 == n) ? 0 : k + 1;
-  const int oc = (1 - colour) * half;
-  const int row = (k * n + j) * n;
-  const int c = row + colour * half + p0;                // own pair
-  const int xo = row + oc + p0;                          // other half, same positions
-  int xe = sigma ? p0 + 2 : p0 - 1;                      // the extra x neighbour
-  if (xe < 0) xe += half;
-  if (xe >= half) xe -= half;
-  xe += row + oc;
-  const int ym = (k * n + jm) * n + oc + p0, yp = (k * n + jp) * n + oc + p0;
-  const int zm = (km * n + j) * n + oc + p0, zp = (kp * n + j) * n + oc + p0;
-  float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f}, s2[2] = {0.f, 0.f};
-  if (!ZERO) {
-    const float* f[3] = {d1, d2, d3};
-    float* acc[3] = {s0, s1, s2};
-#pragma unroll
-    for (int q3 = 0; q3 < 3; ++q3) {
-      const float* v = f[q3];
-      const float2 a = __ldg(reinterpret_cast<const float2*>(v + xo));
-      const float e = __ldg(v + xe);
-      const float2 y0 = __ldg(reinterpret_cast<const float2*>(v + ym));
-      const float2 y1 = __ldg(reinterpret_cast<const float2*>(v + yp));
-      const float2 z0 = __ldg(reinterpret_cast<const float2*>(v + zm));
-      const float2 z1 = __ldg(reinterpret_cast<const float2*>(v + zp));
-      // cell p0: (xm, xp) = sigma ? (a.x, a.y) : (e, a.x); cell p0+1: sigma ? (a.y, e) : (a.x, a.y)
-      const float xm0 = sigma ? a.x : e, xp0 = sigma ? a.y : a.x;
-      const float xm1 = sigma ? a.y : a.x, xp1 = sigma ? e : a.y;
-      acc[q3][0] = ((xm0 + xp0) + (y0.x + y1.x)) + (z0.x + z1.x);
-      acc[q3][1] = ((xm1 + xp1) + (y0.y + y1.y)) + (z0.y + z1.y);
-    }
-  }
-  const float2 qq = __ldg(reinterpret_cast<const float2*>(q + c));
-  const float2 ra = __ldg(reinterpret_cast<const float2*>(r1 + c));
-  const float2 rb = __ldg(reinterpret_cast<const float2*>(r2 + c));
-  const float2 rc = __ldg(reinterpret_cast<const float2*>(r3 + c));
-  float2 dp, dm, dw;
-  lin_point(L, s0[0], s1[0], s2[0], qq.x, ra.x, rb.x, rc.x, dp.x, dm.x, dw.x);
-  lin_point(L, s0[1], s1[1], s2[1], qq.y, ra.y, rb.y, rc.y, dp.y, dm.y, dw.y);
-  *reinterpret_cast<float2*>(d1 + c) = dp;
-  *reinterpret_cast<float2*>(d2 + c) = dm;
-  *reinterpret_cast<float2*>(d3 + c) = dw;
+  if (p >= n >> 1 || j >= n) return;
+  const size_t c = off + (size_t)(k * n + j) * n + p;
+  const float2 z = f2_all(0.f);
+  float2 x[3];
+  lin_point2(L, z, z, z, ldg2(q + c), ldg2(r1 + c), ldg2(r2 + c), ldg2(r3 + c), x[0], x[1], x[2]);
+  *reinterpret_cast<float2*>(d1 + c) = x[0];
+  *reinterpret_cast<float2*>(d2 + c) = x[1];
+  *reinterpret_cast<float2*>(d3 + c) = x[2];
 }
 
 // One damped collective Jacobi sweep on J d = r, d -> t (split layout).
@@ -1322,79 +1444,94 @@ __global__ void k_lin_jacobi32(LvlF L, float w, const float* __restrict__ d1,
 }
 
 
-// The same sweep with two adjacent cells of one half-row per thread (n a
-// multiple of 4): the neighbour pattern of k_lin_smooth32x2 for the pair's
-// colour, own d, r, q and the results as float2.
-template <bool ZERO>
-__global__ void k_lin_jacobi32x2(LvlF L, float w, const float* __restrict__ d1,
-                                 const float* __restrict__ d2, const float* __restrict__ d3,
-                                 float* __restrict__ t1, float* __restrict__ t2,
-                                 float* __restrict__ t3, const float* __restrict__ r1,
-                                 const float* __restrict__ r2, const float* __restrict__ r3,
-                                 const float* __restrict__ q) {
+// The marching sweep: both colours of two positions per thread.
+__global__ void __launch_bounds__(128, 4) k_lin_jacobi32m(
+    LvlF L, float w, int zc, const float* __restrict__ d1, const float* __restrict__ d2,
+    const float* __restrict__ d3, float* __restrict__ t1, float* __restrict__ t2,
+    float* __restrict__ t3, const float* __restrict__ r1, const float* __restrict__ r2,
+    const float* __restrict__ r3, const float* __restrict__ q) {
   pdl_wait();
   pdl_trigger();
-  const int n = L.n, half = n >> 1;
+  const int n = L.n, half = n >> 1, nn = n * n;
+  const MarchCell M(n, zc);
+  if (!M.on) return;
+  const float* const d[3] = {d1 + M.moff, d2 + M.moff, d3 + M.moff};
+  float* const t[3] = {t1 + M.moff, t2 + M.moff, t3 + M.moff};
+  const float* const rq[4] = {r1 + M.moff, r2 + M.moff, r3 + M.moff, q + M.moff};
+  const float2 ww = f2_all(w);
+  float2 zm[3][2], zc_[3][2];
+  const size_t gm = (size_t)(M.k0 == 0 ? n - 1 : M.k0 - 1) * nn;
+#pragma unroll
+  for (int f = 0; f < 3; ++f)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      zm[f][c] = ldg2(d[f] + gm + c * half + M.c);
+      zc_[f][c] = ldg2(d[f] + (size_t)M.k0 * nn + c * half + M.c);
+    }
+#pragma unroll 1
+  for (int k = M.k0; k < M.k1; ++k) {
+    const size_t g = (size_t)k * nn, gp = (size_t)(k + 1 == n ? 0 : k + 1) * nn;
+    const bool sg = (M.j + k) & 1;                   // of colour 0; colour 1 has the other
+    float2 v[4][2], sum[3][2], zp[3][2];
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) v[f][c] = ldg2(rq[f] + g + c * half + M.c);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) zp[f][c] = ldg2(d[f] + gp + c * half + M.c);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const bool s = sg != (c != 0);
+        const float* const o = d[f] + g + (1 - c) * half;
+        sum[f][c] = nbsum2(zc_[f][1 - c], __ldg(o + (s ? M.xr : M.xl)), s, ldg2(o + M.ym),
+                           ldg2(o + M.yp), zm[f][1 - c], zp[f][1 - c]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float2 x[3];
+      lin_point2(L, sum[0][c], sum[1][c], sum[2][c], v[3][c], v[0][c], v[1][c], v[2][c], x[0],
+                 x[1], x[2]);
+#pragma unroll
+      for (int f = 0; f < 3; ++f)
+        *reinterpret_cast<float2*>(t[f] + g + c * half + M.c) =
+            f2_fma(ww, f2_sub(x[f], zc_[f][c]), zc_[f][c]);
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        zm[f][c] = zc_[f][c];
+        zc_[f][c] = zp[f][c];
+      }
+  }
+}
+
+// The first sweep from d = 0 (n a multiple of 4): nothing is read from d.
+__global__ void k_lin_jacobi32_zero(LvlF L, float w, float* __restrict__ t1,
+                                    float* __restrict__ t2, float* __restrict__ t3,
+                                    const float* __restrict__ r1, const float* __restrict__ r2,
+                                    const float* __restrict__ r3, const float* __restrict__ q) {
+  pdl_wait();
+  pdl_trigger();
+  const int n = L.n;
   const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z;
   const size_t off = (size_t)member_of(k, n) * n * n * n;
   if (x >= n || j >= n) return;
-  d1 += off, d2 += off, d3 += off, t1 += off, t2 += off, t3 += off;
-  r1 += off, r2 += off, r3 += off, q += off;
-  const int colour = x >= half, p0 = x - colour * half;
-  const int sigma = (j + k + colour) & 1;
-  const int jm = (j == 0) ? n - 1 : j - 1, jp = (j + 1 == n) ? 0 : j + 1;
-  const int km = (k == 0) ? n - 1 : k - 1, kp = (k + 1 == n) ? 0 : k + 1;
-  const int oc = (1 - colour) * half;
-  const int row = (k * n + j) * n;
-  const int c = row + colour * half + p0;
-  const int xo = row + oc + p0;
-  int xe = sigma ? p0 + 2 : p0 - 1;
-  if (xe < 0) xe += half;
-  if (xe >= half) xe -= half;
-  xe += row + oc;
-  const int ym = (k * n + jm) * n + oc + p0, yp = (k * n + jp) * n + oc + p0;
-  const int zm = (km * n + j) * n + oc + p0, zp = (kp * n + j) * n + oc + p0;
-  float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f}, s2[2] = {0.f, 0.f};
-  float2 o0 = make_float2(0.f, 0.f), o1 = o0, o2 = o0;
-  if (!ZERO) {
-    const float* f[3] = {d1, d2, d3};
-    float* acc[3] = {s0, s1, s2};
-#pragma unroll
-    for (int q3 = 0; q3 < 3; ++q3) {
-      const float* v = f[q3];
-      const float2 a = __ldg(reinterpret_cast<const float2*>(v + xo));
-      const float e = __ldg(v + xe);
-      const float2 y0 = __ldg(reinterpret_cast<const float2*>(v + ym));
-      const float2 y1 = __ldg(reinterpret_cast<const float2*>(v + yp));
-      const float2 z0 = __ldg(reinterpret_cast<const float2*>(v + zm));
-      const float2 z1 = __ldg(reinterpret_cast<const float2*>(v + zp));
-      const float xm0 = sigma ? a.x : e, xp0 = sigma ? a.y : a.x;
-      const float xm1 = sigma ? a.y : a.x, xp1 = sigma ? e : a.y;
-      acc[q3][0] = ((xm0 + xp0) + (y0.x + y1.x)) + (z0.x + z1.x);
-      acc[q3][1] = ((xm1 + xp1) + (y0.y + y1.y)) + (z0.y + z1.y);
-    }
-    o0 = __ldg(reinterpret_cast<const float2*>(d1 + c));
-    o1 = __ldg(reinterpret_cast<const float2*>(d2 + c));
-    o2 = __ldg(reinterpret_cast<const float2*>(d3 + c));
-  }
-  const float2 qq = __ldg(reinterpret_cast<const float2*>(q + c));
-  const float2 ra = __ldg(reinterpret_cast<const float2*>(r1 + c));
-  const float2 rb = __ldg(reinterpret_cast<const float2*>(r2 + c));
-  const float2 rc = __ldg(reinterpret_cast<const float2*>(r3 + c));
-  float2 dp, dm, dw;
-  lin_point(L, s0[0], s1[0], s2[0], qq.x, ra.x, rb.x, rc.x, dp.x, dm.x, dw.x);
-  lin_point(L, s0[1], s1[1], s2[1], qq.y, ra.y, rb.y, rc.y, dp.y, dm.y, dw.y);
-  *reinterpret_cast<float2*>(t1 + c) =
-      make_float2(fmaf(w, dp.x - o0.x, o0.x), fmaf(w, dp.y - o0.y, o0.y));
-  *reinterpret_cast<float2*>(t2 + c) =
-      make_float2(fmaf(w, dm.x - o1.x, o1.x), fmaf(w, dm.y - o1.y, o1.y));
-  *reinterpret_cast<float2*>(t3 + c) =
-      make_float2(fmaf(w, dw.x - o2.x, o2.x), fmaf(w, dw.y - o2.y, o2.y));
+  const size_t c = off + (size_t)(k * n + j) * n + x;
+  const float2 z = f2_all(0.f), ww = f2_all(w);
+  float2 d[3];
+  lin_point2(L, z, z, z, ldg2(q + c), ldg2(r1 + c), ldg2(r2 + c), ldg2(r3 + c), d[0], d[1], d[2]);
+  *reinterpret_cast<float2*>(t1 + c) = f2_fma(ww, d[0], z);
+  *reinterpret_cast<float2*>(t2 + c) = f2_fma(ww, d[1], z);
+  *reinterpret_cast<float2*>(t3 + c) = f2_fma(ww, d[2], z);
 }
 
-// The colour-1 pass of k_lin_smooth32x2 with the defect correction u += d
+// The colour-1 pass of k_lin_smooth32m with the defect correction u += d
 // folded in, for the last pass of a correction's last V-cycle on the finest
 // level: d is not needed after it, so the pass adds its new colour-1 values
 // and the colour-0 values it reads as x neighbours to the FP64 state instead
@@ -1405,7 +1542,7 @@ __global__ void k_lin_jacobi32x2(LvlF L, float w, const float* __restrict__ d1,
 // component.  Same sums and solve as the pass, same u + f2d(d) as
 // k_correct64: u equals the two launches bit for bit.  d's colour-1 cells
 // are left as they were.
-__global__ void k_lin_smooth32x2_correct(LvlF L, const float* __restrict__ d1,
+__global__ void k_lin_smooth32_correct(LvlF L, const float* __restrict__ d1,
                                          const float* __restrict__ d2,
                                          const float* __restrict__ d3,
                                          const float* __restrict__ r1,
@@ -2000,8 +2137,8 @@ dim3 prolong_grid(int nc, int zc, int comps_members) {
 // halo in shared memory and runs that pass from there: the prolonged values
 // never go to global memory, and a launch goes.  Every value is formed with
 // the operations of k_prolong_add32 in its order (z, then y, then x, the
-// 1/64 scale, then the old value) and of k_lin_jacobi32x2 /
-// k_lin_smooth32x2 (sums ((xm + xp) + (ym + yp)) + (zm + zp), lin_point),
+// 1/64 scale, then the old value) and of k_lin_jacobi32m /
+// k_lin_smooth32m (sums ((xm + xp) + (ym + yp)) + (zm + zp), lin_point),
 // so the result equals the two launches bit for bit.
 //
 // A block owns a tile of kPsTX x TY x TZ fine cells in natural order (n a
@@ -3316,6 +3453,7 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
   const int64_t cells = (int64_t)n * n * n * nb;
   const bool pairs = n % 4 == 0;                // two cells per thread, float2 moves
   const Launch3 g = launch3(pairs ? n / 2 : n, n, n * nb);
+  const March mg = march(n, nb);
   float* src[3] = {d[0], d[1], d[2]};
   float* dst[3] = {t[0], t[1], t[2]};
   if (in_t)
@@ -3327,9 +3465,12 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
   cudaError_t e = cudaSuccess;
   while (done < sweeps && e == cudaSuccess) {
     const bool z = zero_init && done == 0;
-    if (pairs)
-      e = launch_k(pdl, z ? k_lin_jacobi32x2<true> : k_lin_jacobi32x2<false>, g.grid, g.block, 0,
-                   st, L, w, src[0], src[1], src[2], dst[0], dst[1], dst[2], r[0], r[1], r[2], q);
+    if (pairs && z)
+      e = launch_k(pdl, k_lin_jacobi32_zero, g.grid, g.block, 0, st, L, w, dst[0], dst[1], dst[2],
+                   r[0], r[1], r[2], q);
+    else if (pairs)
+      e = launch_k(pdl, k_lin_jacobi32m, mg.grid, mg.block, 0, st, L, w, mg.zc, src[0], src[1],
+                   src[2], dst[0], dst[1], dst[2], r[0], r[1], r[2], q);
     else
       e = launch_k(pdl, z ? k_lin_jacobi32<true> : k_lin_jacobi32<false>, g.grid, g.block, 0,
                    st, L, w, src[0], src[1], src[2], dst[0], dst[1], dst[2], r[0], r[1], r[2], q);
@@ -3354,9 +3495,14 @@ cudaError_t rb_pass32(const Ctx32& c, int l, int colour, bool zero) {
   const float* q = c.mx->q[l];
   const bool pairs = L.n % 4 == 0;              // two cells per thread, float2 moves
   const Launch3 g = launch3(pairs ? L.n / 4 : L.n / 2, L.n, L.n * c.nb);
-  if (pairs)
-    return launch_k(c.pr == nullptr, zero ? k_lin_smooth32x2<true> : k_lin_smooth32x2<false>,
-                    g.grid, g.block, 0, c.st, L, colour, d[0], d[1], d[2], r[0], r[1], r[2], q);
+  if (pairs && zero)                            // a zero start begins with colour 0
+    return launch_k(c.pr == nullptr, k_lin_smooth32_zero, g.grid, g.block, 0, c.st, L, d[0], d[1],
+                    d[2], r[0], r[1], r[2], q);
+  if (pairs) {
+    const March mg = march(L.n, c.nb);
+    return launch_k(c.pr == nullptr, k_lin_smooth32m, mg.grid, mg.block, 0, c.st, L, colour, mg.zc,
+                    d[0], d[1], d[2], r[0], r[1], r[2], q);
+  }
   return launch_k(c.pr == nullptr, zero ? k_lin_smooth32<true> : k_lin_smooth32<false>, g.grid,
                   g.block, 0, c.st, L, colour, d[0], d[1], d[2], r[0], r[1], r[2], q);
 }
@@ -3367,7 +3513,7 @@ cudaError_t rb_pass32_correct(const Ctx32& c, int l) {
   float* const* d = c.mx->d[l];
   float* const* r = c.mx->r[l];
   const Launch3 g = launch3(L.n / 4, L.n, L.n * c.nb);
-  return launch_k(c.pr == nullptr, k_lin_smooth32x2_correct, g.grid, g.block, 0, c.st, L,
+  return launch_k(c.pr == nullptr, k_lin_smooth32_correct, g.grid, g.block, 0, c.st, L,
                   (const float*)d[0], (const float*)d[1], (const float*)d[2], (const float*)r[0],
                   (const float*)r[1], (const float*)r[2], (const float*)c.mx->q[l], c.fold_u[0],
                   c.fold_u[1], c.fold_u[2]);
