@@ -3444,19 +3444,18 @@ struct Ctx32 {
   double* const* fold_u = nullptr;   // FP64 state the finest level's last pass adds d to
 };
 
-// `sweeps` damped Jacobi sweeps d -> t -> d ...; the result ends in d.
-// in_t: the current iterate is in t (the sweeps run t -> d -> t ...).
+// `sweeps` damped Jacobi sweeps d -> t -> d ...; *in_t: whether the iterate is
+// in t, on entry and on return.
 cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* const* d,
                      float* const* t, float* const* r, const float* q, cudaStream_t st,
-                     bool pdl, int nb = 1, bool in_t = false) {
+                     bool pdl, int nb, bool* in_t) {
   const int n = L.n;
-  const int64_t cells = (int64_t)n * n * n * nb;
   const bool pairs = n % 4 == 0;                // two cells per thread, float2 moves
   const Launch3 g = launch3(pairs ? n / 2 : n, n, n * nb);
   const March mg = march(n, nb);
   float* src[3] = {d[0], d[1], d[2]};
   float* dst[3] = {t[0], t[1], t[2]};
-  if (in_t)
+  if (*in_t)
     for (int c = 0; c < 3; ++c) {
       src[c] = t[c];
       dst[c] = d[c];
@@ -3481,9 +3480,21 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
       dst[c] = x;
     }
   }
-  if (e == cudaSuccess && src[0] != d[0])
-    e = launch_k(pdl, k_copy3, dim3(grid_for(cells)), dim3(kThreads), 0, st, (int)cells, src[0],
-                 src[1], src[2], d[0], d[1], d[2]);
+  *in_t = src[0] != d[0];
+  return e;
+}
+
+// jacobi32 on level l of a cycle: where the result is in t, d and t change
+// places (the cycle's own pointers), so no copy follows an odd count.
+cudaError_t jacobi_level32(const Ctx32& c, int l, int sweeps, bool zero_init, bool in_t) {
+  cudaError_t e = jacobi32(c.L[l], sweeps, c.w, zero_init, c.mx->d[l], c.mx->t[l], c.mx->r[l],
+                           c.mx->q[l], c.st, c.pr == nullptr, c.nb, &in_t);
+  if (in_t)
+    for (int f = 0; f < 3; ++f) {
+      float* const x = c.mx->d[l][f];
+      c.mx->d[l][f] = c.mx->t[l][f];
+      c.mx->t[l][f] = x;
+    }
   return e;
 }
 
@@ -3531,16 +3542,11 @@ bool correction_folds(const Ctx32& c) {
 // `sweeps` post- (or pre-) smoothing sweeps on level l; fold: the last
 // colour-1 pass adds the result to c.fold_u (red-black, n % 4 == 0).
 cudaError_t smooth32(const Ctx32& c, int l, int sweeps, bool zero_init, bool fold = false) {
-  const LvlF& L = c.L[l];
-  float* const* d = c.mx->d[l];
-  float* const* r = c.mx->r[l];
-  const float* q = c.mx->q[l];
   if (sweeps <= 0) return cudaSuccess;
   prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
   if (c.kind[l] == PFC_SWEEP_JACOBI) {
     const int js = sweeps * (l == 0 ? c.jfactor0 : c.jfactor);
-    cudaError_t e =
-        jacobi32(L, js, c.w, zero_init, d, c.mx->t[l], r, q, c.st, c.pr == nullptr, c.nb);
+    cudaError_t e = jacobi_level32(c, l, js, zero_init, false);
     prof_end(c.pr, PFC_K_LIN_SMOOTH, l, js, c.st);
     return e;
   }
@@ -3559,9 +3565,20 @@ cudaError_t smooth32(const Ctx32& c, int l, int sweeps, bool zero_init, bool fol
   return e;
 }
 
-// Whether the prolongation into a level of n^3 cells fuses with the first
+// Whether the prolongation into a level of n^3 cells can fuse with the first
 // of `sweeps` post-smoothing sweeps (k_lin_prolong_sweep32's tiles).
 bool prolong_fuses(int n, int sweeps) { return sweeps > 0 && n >= kPsTX && n % kPsTX == 0; }
+
+// Whether it pays: the fused kernel saves a launch and 24 B a cell, but forms
+// every value of its tile's halo again in shared memory, so it wins on small
+// levels only.  In-graph us, fused / the two launches: d += P e 32^3 2.7 /
+// 3.8, 10 x 32^3 6.9 / 8.7, 28 x 32^3 15.2 / 15.8, 42 x 32^3 22.0 / 20.1, 64^3
+// 6.8 / 5.8, 128^3 30.8 / 21.0, 256^3 236 / 174, 42 x 64^3 145 / 119; d = P e
+// (d is not read) 64^3 4.6 / 7.2, 96^3 10.1 / 11.7, 4 x 64^3 11.8 / 12.0,
+// 128^3 22.5 / 20.5, 256^3 162 / 142.
+bool prolong_fuse_pays(int n, int members, bool assign) {
+  return (int64_t)n * n * n * members <= (1 << 20) && (assign || n < 64);
+}
 
 template <int TY, int TZ>
 cudaError_t launch_prolong_sweep(const Ctx32& c, int l, bool jacobi, bool assign) {
@@ -3592,8 +3609,7 @@ cudaError_t prolong_smooth32(const Ctx32& c, int l, bool assign, int sweeps) {
   if (jacobi) {
     // the first sweep left its result in t
     prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
-    e = jacobi32(c.L[l], sweeps - 1, c.w, false, c.mx->d[l], c.mx->t[l], c.mx->r[l], c.mx->q[l],
-                 c.st, c.pr == nullptr, c.nb, true);
+    e = jacobi_level32(c, l, sweeps - 1, false, true);
     prof_end(c.pr, PFC_K_LIN_SMOOTH, l, sweeps - 1, c.st);
     return e;
   }
@@ -3854,7 +3870,8 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
   // pass formed every colour-1 value of its tile and halo per cell (25 us
   // per launch at 128^3 against 6.1 + 6.5 us for the prolongation's
   // coarse-column carry and the plain pass)
-  if (c.kind[l] == PFC_SWEEP_JACOBI && prolong_fuses(L.n, post))
+  if (c.kind[l] == PFC_SWEEP_JACOBI && prolong_fuses(L.n, post) &&
+      prolong_fuse_pays(L.n, c.nb, dzero))
     return prolong_smooth32(c, l, dzero, post);
   const int pz = prolong_planes(nc, 3 * c.nb);
   // a red-black post-smoothing pass of colour 0 comes next: it recomputes
@@ -4179,6 +4196,14 @@ cudaError_t launch_prolong32(int n, bool assign, bool skip0, const float* e1, co
                   dim3(kPrTI * kPrTJ), 0, st, n, pz, e1, e2, e3, d1, d2, d3);
 }
 
+// The result of an odd number of Jacobi sweeps from t to the caller's d.
+static cudaError_t launch_copy3(int n, float* const* t, float* d1, float* d2, float* d3,
+                                cudaStream_t st) {
+  const int64_t cells = (int64_t)n * n * n;
+  return launch_k(true, k_copy3, dim3(grid_for(cells)), dim3(kThreads), 0, st, (int)cells,
+                  (const float*)t[0], (const float*)t[1], (const float*)t[2], d1, d2, d3);
+}
+
 cudaError_t launch_lin_smooth32(const Lvl& L, int sweeps, bool zero_init, float* d1,
                                 float* d2, float* d3, const float* r1, const float* r2,
                                 const float* r3, const float* q, cudaStream_t st) {
@@ -4263,7 +4288,9 @@ cudaError_t launch_lin_prolong_smooth32(const Lvl& L, int kind, bool assign, flo
   c.jfactor0 = 1;
   c.st = st;
   c.pr = nullptr;
-  return prolong_smooth32(c, 0, assign, 1);
+  const cudaError_t e = prolong_smooth32(c, 0, assign, 1);
+  if (e != cudaSuccess || mx.d[0][0] == d1) return e;
+  return launch_copy3(L.n, mx.d[0], d1, d2, d3, st);
 }
 
 cudaError_t launch_lin_jacobi32(const Lvl& L, int sweeps, float w, bool zero_init,
@@ -4273,7 +4300,9 @@ cudaError_t launch_lin_jacobi32(const Lvl& L, int sweeps, float w, bool zero_ini
   float* d[3] = {d1, d2, d3};
   float* t[3] = {t1, t2, t3};
   float* r[3] = {(float*)r1, (float*)r2, (float*)r3};
-  return jacobi32(to_f32(L), sweeps, w, zero_init, d, t, r, q, st, true);
+  bool in_t = false;
+  const cudaError_t e = jacobi32(to_f32(L), sweeps, w, zero_init, d, t, r, q, st, true, 1, &in_t);
+  return e == cudaSuccess && in_t ? launch_copy3(L.n, t, d1, d2, d3, st) : e;
 }
 
 cudaError_t launch_correct_df(int n, float2* u1, float2* u2, float2* u3, const float* d1,
@@ -4366,6 +4395,8 @@ namespace {
 // then p.inner_cycles V-cycles from d = 0.  u (FP64 state, or nullptr): where
 // correction_folds holds, the last V-cycle's last pass adds d to u (*folded
 // set), and the caller's u += d launch goes.
+// mx: the caller's own copy of the buffers' pointers (a cycle may leave d and t
+// of a level exchanged).
 cudaError_t mixed_vcycles(MixedBufs& mx, const pfc_params& p, int nl, const int* sizes,
                           cudaStream_t st, Prof* pr, int members, double tau_scale,
                           double* const* u, bool* folded) {
@@ -4419,9 +4450,10 @@ cudaError_t mixed_vcycles(MixedBufs& mx, const pfc_params& p, int nl, const int*
 
 }  // namespace
 
-cudaError_t mixed_enqueue_correction(MixedBufs& mx, const pfc_params& p, int nl,
+cudaError_t mixed_enqueue_correction(const MixedBufs& bufs, const pfc_params& p, int nl,
                                      const int* sizes, double* const u[3], cudaStream_t st,
                                      Prof* pr, int members, double tau_scale) {
+  MixedBufs mx = bufs;
   bool folded = false;
   cudaError_t e = mixed_vcycles(mx, p, nl, sizes, st, pr, members, tau_scale, u, &folded);
   if (e == cudaSuccess && !folded) {
@@ -4433,9 +4465,10 @@ cudaError_t mixed_enqueue_correction(MixedBufs& mx, const pfc_params& p, int nl,
   return e;
 }
 
-cudaError_t mixed_enqueue_correction(MixedBufs& mx, const pfc_params& p, int nl,
+cudaError_t mixed_enqueue_correction(const MixedBufs& bufs, const pfc_params& p, int nl,
                                      const int* sizes, float2* const u[3], cudaStream_t st,
                                      Prof* pr) {
+  MixedBufs mx = bufs;
   bool folded = false;
   cudaError_t e = mixed_vcycles(mx, p, nl, sizes, st, pr, 1, 1.0, nullptr, &folded);
   if (e == cudaSuccess) {

@@ -115,10 +115,10 @@ cudaError_t mixed_enqueue_defect(MixedBufs& mx, const Lvl& L0, float2* const u[3
 // One defect correction after mixed_enqueue_defect: q restricted to every
 // level, p.inner_cycles FP32 V-cycles on J d = r from d = 0, then u += d in
 // FP64 (PFC_MIXED) or double-float (PFC_MIXED_DF).
-cudaError_t mixed_enqueue_correction(MixedBufs& mx, const pfc_params& p, int nl,
+cudaError_t mixed_enqueue_correction(const MixedBufs& bufs, const pfc_params& p, int nl,
                                      const int* sizes, double* const u[3], cudaStream_t st,
                                      Prof* pr, int members = 1, double tau_scale = 1.0);
-cudaError_t mixed_enqueue_correction(MixedBufs& mx, const pfc_params& p, int nl,
+cudaError_t mixed_enqueue_correction(const MixedBufs& bufs, const pfc_params& p, int nl,
                                      const int* sizes, float2* const u[3], cudaStream_t st,
                                      Prof* pr);
 
