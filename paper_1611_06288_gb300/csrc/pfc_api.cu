@@ -301,11 +301,11 @@ int smooth_level(pfc_ctx* c, int l, const Level64& lv, int sweeps) {
     PFC_TIMED(pr, PFC_K_SMOOTH, l, js, st,
               launch_jacobi(lv.L, c->p.smoother, js, c->p.jacobi_weight, lv.u[0], lv.u[1],
                             lv.u[2], lv.t[0], lv.t[1], lv.t[2], lv.S[0], lv.S[1], lv.S[2],
-                            lv.b, st));
+                            lv.b, st, pr->mask == 0));
   } else {
     PFC_TIMED(pr, PFC_K_SMOOTH, l, 2 * sweeps, st,
               launch_smooth(lv.L, c->p.smoother, sweeps, lv.u[0], lv.u[1], lv.u[2], lv.S[0],
-                            lv.S[1], lv.S[2], lv.b, st));
+                            lv.S[1], lv.S[2], lv.b, st, pr->mask == 0));
   }
   return PFC_OK;
 }
@@ -318,7 +318,7 @@ int vcycle64(pfc_ctx* c, int l, const Level64& lv) {
     PFC_TIMED(pr, PFC_K_COARSE_SOLVE, l, 1, st,
               launch_coarse_solve(lv.L, lin, lv.kind, c->p.jacobi_weight, 400, lv.u[0],
                                   lv.u[1], lv.u[2], lv.t[0], lv.t[1], lv.t[2], lv.S[0],
-                                  lv.S[1], lv.S[2], lv.b, st));
+                                  lv.S[1], lv.S[2], lv.b, st, pr->mask == 0));
     return PFC_OK;
   }
   Level64& cl = c->lev[l + 1];
@@ -327,18 +327,16 @@ int vcycle64(pfc_ctx* c, int l, const Level64& lv) {
   PFC_TIMED(pr, PFC_K_RESIDUAL_RESTRICT, l, 1, st,
             launch_residual_restrict(lv.L, lv.u[0], lv.u[1], lv.u[2], lv.S[0], lv.S[1],
                                      lv.S[2], lv.b, cl.S[0], cl.S[1], cl.S[2], cl.u[0],
-                                     cl.u[1], cl.u[2], cl.w[0], cl.w[1], cl.w[2], st));
+                                     cl.u[1], cl.u[2], cl.w[0], cl.w[1], cl.w[2], st,
+                                     pr->mask == 0));
   PFC_TIMED(pr, PFC_K_COARSE_SOURCE, l + 1, 1, st,
             launch_coarse_source(cl.L, cl.u[0], cl.u[1], cl.u[2], cl.b, cl.S[0], cl.S[1],
-                                 cl.S[2], st));
+                                 cl.S[2], st, pr->mask == 0));
   int rc = vcycle64(c, l + 1, cl);
   if (rc) return rc;
-  prof_begin(pr, PFC_K_PROLONG, st);
-  PFC_CUDA(launch_coarse_diff(cl.n, cl.u[0], cl.u[1], cl.u[2], cl.w[0], cl.w[1], cl.w[2],
-                              st));
-  PFC_CUDA(launch_prolong_add(lv.n, cl.w[0], cl.w[1], cl.w[2], lv.u[0], lv.u[1], lv.u[2],
-                              st));
-  prof_end(pr, PFC_K_PROLONG, l, 2, st);
+  PFC_TIMED(pr, PFC_K_PROLONG, l, 1, st,
+            launch_prolong_add(lv.n, cl.u[0], cl.u[1], cl.u[2], cl.w[0], cl.w[1], cl.w[2],
+                               lv.u[0], lv.u[1], lv.u[2], st, pr->mask == 0));
   return smooth_level(c, l, lv, c->p.nu2);
 }
 
@@ -442,7 +440,7 @@ int enqueue_residual_decide(pfc_ctx* c, const Level64& lv, cudaGraphConditionalH
     PFC_TIMED(&c->prof, PFC_K_RESIDUAL_NORM, 0, 2, st,
               launch_residual_norm2(lv.L, lv.u[0], lv.u[1], lv.u[2], lv.S[0], lv.S[1],
                                     lv.S[2], lv.b, c->partials, c->dout, st,
-                                    c->lap[c->ia]));
+                                    c->lap[c->ia], c->prof.mask == 0, &da, &decided));
   }
   // a residual that took the decision in its reduction needs no launch of it
   return decided ? PFC_OK : enqueue_decide(c, h, use_handle, first);
@@ -505,7 +503,8 @@ int enqueue_pre(pfc_ctx* c, const Level64& lv, cudaGraphConditionalHandle h, int
     const double* fine = lv.b;
     for (int l = 1; l < c->nl; ++l) {
       PFC_TIMED(pr, PFC_K_RESTRICT, l - 1, 1, c->st,
-                launch_restrict(c->sizes[l - 1], fine, c->lev[l].b, c->st));
+                launch_restrict(c->sizes[l - 1], fine, c->lev[l].b, c->st,
+                                c->prof.mask == 0));
       fine = c->lev[l].b;
     }
   }
@@ -1620,11 +1619,7 @@ int pfc_op_prolong_correct(int n, const double* vc1, const double* vc2, const do
                            double* u1, double* u2, double* u3, void* stream) {
   if (n < 2 || (n & 1) || !vc1 || !vc2 || !vc3 || !wc1 || !wc2 || !wc3 || !u1 || !u2 || !u3)
     return PFC_EINVAL;
-  // e = v - w is formed in place over w, then interpolated and added.
-  cudaStream_t st = (cudaStream_t)stream;
-  PFC_CUDA(launch_coarse_diff(n / 2, vc1, vc2, vc3, (double*)wc1, (double*)wc2,
-                              (double*)wc3, st));
-  PFC_CUDA(launch_prolong_add(n, wc1, wc2, wc3, u1, u2, u3, st));
+  PFC_CUDA(launch_prolong_add(n, vc1, vc2, vc3, wc1, wc2, wc3, u1, u2, u3, (cudaStream_t)stream));
   return PFC_OK;
 }
 

@@ -15,6 +15,16 @@ inline unsigned grid_for(int64_t work, int threads = kThreads) {
   return (unsigned)((work + threads - 1) / threads);
 }
 
+// Threads per block of a grid of `work` threads: 256, halved (to 32) while the
+// blocks would not reach every SM.  The small levels are bound by one SM's
+// FP64 rate (2 lanes a clock: a red-black pass of 8^3 cells took 4.6 us in one
+// block of 256) and by launches.
+inline int block_for(int64_t work) {
+  int t = kThreads;
+  while (t > 32 && work < (int64_t)152 * t) t >>= 1;
+  return t;
+}
+
 __device__ __forceinline__ void cell_of(int64_t t, int n, int& i, int& j, int& k) {
   i = (int)(t % n);
   const int64_t r = t / n;
@@ -153,6 +163,8 @@ __global__ void k_smooth_colour(Lvl L, int colour, double* phi, double* mu, doub
                                 const double* __restrict__ S2,
                                 const double* __restrict__ S3,
                                 const double* __restrict__ b) {
+  pdl_wait();
+  pdl_trigger();
   const int n = L.n, half = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)half * n * n) return;
@@ -182,6 +194,8 @@ __global__ void k_jacobi64(Lvl L, double w, const double* __restrict__ phi,
                            double* __restrict__ tw, const double* __restrict__ S1,
                            const double* __restrict__ S2, const double* __restrict__ S3,
                            const double* __restrict__ b) {
+  pdl_wait();
+  pdl_trigger();
   const int n = L.n;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n * n) return;
@@ -220,54 +234,156 @@ __global__ void k_residual(Lvl L, const double* __restrict__ phi,
 }
 
 // ---------------------------------------------------------------------------
-// a3: fused residual + 8-cell restriction of r and u; one thread per coarse
-// cell.  Optionally also stores the restricted u a second time (wc), which the
-// correction step needs after the coarse level has overwritten uc.
+// a3: fused residual + 8-cell restriction of r and u.  Optionally also stores
+// the restricted u a second time (wc), which the correction step needs after
+// the coarse level has overwritten uc.
+//
+// Small grids: eight lanes per coarse cell, one child each, summed by the
+// first lane in the children's order.  (One thread per coarse cell ran the
+// eight residuals one after another: 24 us at every size up to 32^3.)
 // ---------------------------------------------------------------------------
-__global__ void k_residual_restrict(Lvl L, const double* __restrict__ phi,
-                                    const double* __restrict__ mu,
-                                    const double* __restrict__ om,
-                                    const double* __restrict__ S1,
-                                    const double* __restrict__ S2,
-                                    const double* __restrict__ S3,
-                                    const double* __restrict__ b, double* __restrict__ rc1,
-                                    double* __restrict__ rc2, double* __restrict__ rc3,
-                                    double* __restrict__ uc1, double* __restrict__ uc2,
-                                    double* __restrict__ uc3, double* __restrict__ wc1,
-                                    double* __restrict__ wc2, double* __restrict__ wc3) {
+__global__ void k_residual_restrict8(Lvl L, const double* __restrict__ phi,
+                                     const double* __restrict__ mu,
+                                     const double* __restrict__ om,
+                                     const double* __restrict__ S1,
+                                     const double* __restrict__ S2,
+                                     const double* __restrict__ S3,
+                                     const double* __restrict__ b, double* __restrict__ rc1,
+                                     double* __restrict__ rc2, double* __restrict__ rc3,
+                                     double* __restrict__ uc1, double* __restrict__ uc2,
+                                     double* __restrict__ uc3, double* __restrict__ wc1,
+                                     double* __restrict__ wc2, double* __restrict__ wc3) {
+  pdl_wait();
+  pdl_trigger();
+  const int n = L.n, nc = n >> 1;
+  const int64_t cells = (int64_t)nc * nc * nc;
+  const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = x >> 3;
+  const int c = (int)(x & 7);
+  double v[6] = {0, 0, 0, 0, 0, 0};
+  if (t < cells) {                       // whole groups of eight lanes
+    int I, J, K;
+    cell_of(t, nc, I, J, K);
+    const Stencil s = stencil_at(2 * I + (c & 1), 2 * J + ((c >> 1) & 1), 2 * K + (c >> 2), n);
+    residual_at(L, s, phi, mu, om, S1, S2, S3, b, v[0], v[1], v[2]);
+    v[3] = __ldg(phi + s.c);
+    v[4] = __ldg(mu + s.c);
+    v[5] = __ldg(om + s.c);
+  }
+  double a[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+#pragma unroll
+    for (int f = 0; f < 6; ++f) a[f] += __shfl_sync(0xffffffffu, v[f], q, 8);
+  if (t >= cells || c) return;
+  rc1[t] = 0.125 * a[0];
+  rc2[t] = 0.125 * a[1];
+  rc3[t] = 0.125 * a[2];
+  uc1[t] = 0.125 * a[3];
+  uc2[t] = 0.125 * a[4];
+  uc3[t] = 0.125 * a[5];
+  if (wc1) {
+    wc1[t] = 0.125 * a[3];
+    wc2[t] = 0.125 * a[4];
+    wc3[t] = 0.125 * a[5];
+  }
+}
+
+// Sums of one field over the eight children of a coarse cell (in) and over
+// the 24 face neighbours outside them (out).  c0, the children's first cell, is
+// even in x: rows of two cells are one 16-byte load.
+struct BlockAt {
+  int64_t c[4];                          // rows (jj, kk) of the children: first cell
+  int64_t y[4], z[4];                    // rows below / above in y, in z
+  int xm, xp;                            // x offsets of the neighbours beside a row
+  __device__ __forceinline__ BlockAt(int I, int J, int K, int n) {
+    const int i = 2 * I, j = 2 * J, k = 2 * K;
+    const int64_t nn = (int64_t)n * n;
+    const int jm = j == 0 ? n - 1 : j - 1, jp = j + 2 == n ? 0 : j + 2;
+    const int km = k == 0 ? n - 1 : k - 1, kp = k + 2 == n ? 0 : k + 2;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[q] = i + (int64_t)n * (j + (q & 1)) + nn * (k + (q >> 1));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      y[q] = i + (int64_t)n * jm + nn * (k + q);
+      y[2 + q] = i + (int64_t)n * jp + nn * (k + q);
+      z[q] = i + (int64_t)n * (j + q) + nn * km;
+      z[2 + q] = i + (int64_t)n * (j + q) + nn * kp;
+    }
+    xm = i == 0 ? n - 1 : -1;
+    xp = i + 2 == n ? 2 - n : 2;
+  }
+  __device__ __forceinline__ static double2 ld(const double* v, int64_t at) {
+    return __ldg(reinterpret_cast<const double2*>(v + at));
+  }
+  __device__ __forceinline__ void sums(const double* __restrict__ v, double2 (&in)[4],
+                                       double& sin, double& sout) const {
+    sin = sout = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) in[q] = ld(v, c[q]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      sin += in[q].x;
+      sin += in[q].y;
+      const double2 a = ld(v, y[q]), d = ld(v, z[q]);
+      sout += (__ldg(v + c[q] + xm) + __ldg(v + c[q] + xp)) + ((a.x + a.y) + (d.x + d.y));
+    }
+  }
+};
+
+// Large grids, one thread per coarse cell: the Laplacians of the eight
+// children are summed as sum_out - 3 sum_in (the inner faces of the block
+// cancel) and the linear terms of the rows from the sums, which takes 21
+// instead of 40 FP64 operations per fine cell: the pass is bound by the FP64
+// pipe (128^3: 154 -> 87 us).  n even, pointers 16-byte aligned.
+__global__ void __launch_bounds__(128) k_residual_restrict(
+    Lvl L, const double* __restrict__ phi, const double* __restrict__ mu,
+    const double* __restrict__ om, const double* __restrict__ S1, const double* __restrict__ S2,
+    const double* __restrict__ S3, const double* __restrict__ b, double* __restrict__ rc1,
+    double* __restrict__ rc2, double* __restrict__ rc3, double* __restrict__ uc1,
+    double* __restrict__ uc2, double* __restrict__ uc3, double* __restrict__ wc1,
+    double* __restrict__ wc2, double* __restrict__ wc3) {
+  pdl_wait();
+  pdl_trigger();
   const int n = L.n, nc = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nc * nc * nc) return;
   int I, J, K;
   cell_of(t, nc, I, J, K);
-  double a1 = 0, a2 = 0, a3 = 0, v1 = 0, v2 = 0, v3 = 0;
+  const BlockAt B(I, J, K, n);
+  double2 p[4], x[4];
+  double ip, op, im, om_, iw, ow;
+  B.sums(phi, p, ip, op);
+  B.sums(mu, x, im, om_);
+  B.sums(om, x, iw, ow);
+  double s1 = 0, s2 = 0, s3 = 0, f4 = 0;   // f4: 4 sum f(phi, b)
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int i = 2 * I + (c & 1), j = 2 * J + ((c >> 1) & 1), k = 2 * K + (c >> 2);
-    const Stencil s = stencil_at(i, j, k, n);
-    double x, y, z;
-    residual_at(L, s, phi, mu, om, S1, S2, S3, b, x, y, z);
-    a1 += x;
-    a2 += y;
-    a3 += z;
-    v1 += __ldg(phi + s.c);
-    v2 += __ldg(mu + s.c);
-    v3 += __ldg(om + s.c);
+  for (int q = 0; q < 4; ++q) {
+    const double2 v = BlockAt::ld(S1, B.c[q]), w = BlockAt::ld(S2, B.c[q]),
+                  u = BlockAt::ld(S3, B.c[q]);
+    const double2 bb = S1 == b ? v : BlockAt::ld(b, B.c[q]);
+    s1 += v.x + v.y;
+    s2 += w.x + w.y;
+    s3 += u.x + u.y;
+    f4 = fma(p[q].x + bb.x, fma(p[q].x, p[q].x, bb.x * bb.x), f4);
+    f4 = fma(p[q].y + bb.y, fma(p[q].y, p[q].y, bb.y * bb.y), f4);
   }
-  rc1[t] = 0.125 * a1;
-  rc2[t] = 0.125 * a2;
-  rc3[t] = 0.125 * a3;
-  uc1[t] = 0.125 * v1;
-  uc2[t] = 0.125 * v2;
-  uc3[t] = 0.125 * v3;
+  rc1[t] = 0.125 * fma(L.tg, fma(-3.0, im, om_), s1 - ip);
+  rc2[t] = 0.125 * fma(L.g, fma(-3.0, iw, ow), fma(L.c1, ip, fma(0.25, f4, s2 - im)));
+  rc3[t] = 0.125 * fma(L.gh, fma(-3.0, ip, op), s3 - iw);
+  uc1[t] = 0.125 * ip;
+  uc2[t] = 0.125 * im;
+  uc3[t] = 0.125 * iw;
   if (wc1) {
-    wc1[t] = 0.125 * v1;
-    wc2[t] = 0.125 * v2;
-    wc3[t] = 0.125 * v3;
+    wc1[t] = 0.125 * ip;
+    wc2[t] = 0.125 * im;
+    wc3[t] = 0.125 * iw;
   }
 }
 
 __global__ void k_restrict(int n, const double* __restrict__ f, double* __restrict__ c) {
+  pdl_wait();
+  pdl_trigger();
   const int nc = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nc * nc * nc) return;
@@ -290,6 +406,8 @@ __global__ void k_coarse_source(Lvl L, const double* __restrict__ u1,
                                 const double* __restrict__ u3,
                                 const double* __restrict__ bc, double* r1, double* r2,
                                 double* r3) {
+  pdl_wait();
+  pdl_trigger();
   const int n = L.n;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n * n) return;
@@ -303,38 +421,34 @@ __global__ void k_coarse_source(Lvl L, const double* __restrict__ u1,
   r3[s.c] += z;
 }
 
-__global__ void k_coarse_diff(int64_t cells, const double* __restrict__ v1,
-                              const double* __restrict__ v2,
-                              const double* __restrict__ v3, double* w1, double* w2,
-                              double* w3) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= cells) return;
-  w1[t] = v1[t] - w1[t];
-  w2[t] = v2[t] - w2[t];
-  w3[t] = v3[t] - w3[t];
-}
-
 // ---------------------------------------------------------------------------
-// a6: u += P e, P trilinear cell-centred: fine cell 2I+a takes 3/4 of coarse I
-// and 1/4 of coarse I+(a ? 1 : -1) per axis, i.e. weights 27, 9, 3, 1 (/64).
+// a6: u += P (v - w), P trilinear cell-centred: fine cell 2I+a takes 3/4 of
+// coarse I and 1/4 of coarse I+(a ? 1 : -1) per axis, i.e. weights 27, 9, 3, 1
+// (/64); v the coarse solution, w the restricted u it started from.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double interp8(const double* __restrict__ e, int64_t o000,
+__device__ __forceinline__ double interp8(const double* __restrict__ v,
+                                          const double* __restrict__ w, int64_t o000,
                                           int64_t o100, int64_t o010, int64_t o001,
                                           int64_t o110, int64_t o101, int64_t o011,
                                           int64_t o111) {
-  const double g2 = (__ldg(e + o100) + __ldg(e + o010)) + __ldg(e + o001);
-  const double g3 = (__ldg(e + o110) + __ldg(e + o101)) + __ldg(e + o011);
-  double acc = fma(3.0, g3, __ldg(e + o111));
+  const auto e = [&](int64_t o) { return __ldg(v + o) - __ldg(w + o); };
+  const double g2 = (e(o100) + e(o010)) + e(o001);
+  const double g3 = (e(o110) + e(o101)) + e(o011);
+  double acc = fma(3.0, g3, e(o111));
   acc = fma(9.0, g2, acc);
-  acc = fma(27.0, __ldg(e + o000), acc);
+  acc = fma(27.0, e(o000), acc);
   return acc;
 }
 
-__global__ void k_prolong_add(int n, const double* __restrict__ e1,
-                              const double* __restrict__ e2,
-                              const double* __restrict__ e3, double* __restrict__ u1,
-                              double* __restrict__ u2, double* __restrict__ u3) {
-  const int nc = n >> 1;
+// One fine cell and component (blockIdx.y) per thread: the small levels.
+__global__ void k_prolong_add(int n, const double* __restrict__ v1, const double* __restrict__ v2,
+                              const double* __restrict__ v3, const double* __restrict__ w1,
+                              const double* __restrict__ w2, const double* __restrict__ w3,
+                              double* __restrict__ u1, double* __restrict__ u2,
+                              double* __restrict__ u3) {
+  pdl_wait();
+  pdl_trigger();
+  const int nc = n >> 1, f = blockIdx.y;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n * n) return;
   int i, j, k;
@@ -351,10 +465,105 @@ __global__ void k_prolong_add(int n, const double* __restrict__ e1,
   const int64_t o000 = I + yJ + zK, o100 = I2 + yJ + zK, o010 = I + yJ2 + zK,
                 o001 = I + yJ + zK2, o110 = I2 + yJ2 + zK, o101 = I2 + yJ + zK2,
                 o011 = I + yJ2 + zK2, o111 = I2 + yJ2 + zK2;
-  const double w = 1.0 / 64.0;
-  u1[t] = fma(w, interp8(e1, o000, o100, o010, o001, o110, o101, o011, o111), u1[t]);
-  u2[t] = fma(w, interp8(e2, o000, o100, o010, o001, o110, o101, o011, o111), u2[t]);
-  u3[t] = fma(w, interp8(e3, o000, o100, o010, o001, o110, o101, o011, o111), u3[t]);
+  double* const u = f == 0 ? u1 : f == 1 ? u2 : u3;
+  u[t] = fma(1.0 / 64.0,
+             interp8(f == 0 ? v1 : f == 1 ? v2 : v3, f == 0 ? w1 : f == 1 ? w2 : w3, o000, o100,
+                     o010, o001, o110, o101, o011, o111),
+             u[t]);
+}
+
+// Large levels: the interpolation as one-dimensional passes, z then y then x
+// ((3 e_0 + e_-1) / 4 and (3 e_0 + e_+1) / 4 per axis), 31 FP64 operations per
+// eight children and component instead of 64: the pass is bound by the FP64
+// pipe (128^3: 99 -> 44 us).  A block of kPfI x kPfJ threads owns that tile of
+// coarse columns of one component and marches over zc coarse planes; each
+// thread interpolates its own column (and at most one of the tile's halo) in z
+// from values it carries, the tile's columns meet in shared memory (double
+// buffered, one barrier a plane), and each thread then writes its coarse
+// cell's eight children as four 16-byte pairs.  n even, u 16-byte aligned.
+constexpr int kPfI = 32, kPfJ = 4;
+
+__global__ void __launch_bounds__(kPfI * kPfJ) k_prolong_add_tile(
+    int n, int zc, const double* __restrict__ v1, const double* __restrict__ v2,
+    const double* __restrict__ v3, const double* __restrict__ w1, const double* __restrict__ w2,
+    const double* __restrict__ w3, double* __restrict__ u1, double* __restrict__ u2,
+    double* __restrict__ u3) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int W = kPfI + 2, H = kPfJ + 2;
+  __shared__ double sh[2][2][H][W];          // [buffer][child in z][y][x]
+  const int nc = n >> 1, chunks = (nc + zc - 1) / zc;
+  const int f = blockIdx.z / chunks, K0 = (blockIdx.z - f * chunks) * zc, K1 = min(nc, K0 + zc);
+  const double* const v = f == 0 ? v1 : f == 1 ? v2 : v3;
+  const double* const w = f == 0 ? w1 : f == 1 ? w2 : w3;
+  double* const u = f == 0 ? u1 : f == 1 ? u2 : u3;
+  const int tid = threadIdx.x, tx = tid % kPfI, ty = tid / kPfI;
+  const int I = blockIdx.x * kPfI + tx, J = blockIdx.y * kPfJ + ty;
+  const auto wrap = [nc](int x) { return (x + nc) % nc; };
+  // halo column of this thread: the rows above and below the tile with their
+  // corners, then the columns beside it
+  constexpr int kHalo = 2 * W + 2 * kPfJ;
+  static_assert(kHalo <= kPfI * kPfJ, "one halo column per thread at most");
+  int hx = 0, hy = 0;
+  if (tid < 2 * W) {
+    hx = tid < W ? tid : tid - W;
+    hy = tid < W ? 0 : H - 1;
+  } else if (tid < kHalo) {
+    const int r = tid - 2 * W;
+    hx = r < kPfJ ? 0 : W - 1;
+    hy = 1 + (r < kPfJ ? r : r - kPfJ);
+  }
+  const bool halo = tid < kHalo;
+  const int64_t plane = (int64_t)nc * nc;
+  const int64_t oa = (int64_t)wrap(J) * nc + wrap(I);
+  const int64_t oh = (int64_t)wrap(blockIdx.y * kPfJ + hy - 1) * nc +
+                     wrap(blockIdx.x * kPfI + hx - 1);
+  const auto e = [&](int K, int64_t o) {
+    K = K < 0 ? K + nc : K >= nc ? K - nc : K;
+    return __ldg(v + K * plane + o) - __ldg(w + K * plane + o);
+  };
+  double am = e(K0 - 1, oa), ac = e(K0, oa), hm = 0, hc = 0;
+  if (halo) {
+    hm = e(K0 - 1, oh);
+    hc = e(K0, oh);
+  }
+  for (int K = K0; K < K1; ++K) {
+    double (*const s)[H][W] = sh[K & 1];
+    const double ap = e(K + 1, oa);
+    s[0][ty + 1][tx + 1] = fma(3.0, ac, am);
+    s[1][ty + 1][tx + 1] = fma(3.0, ac, ap);
+    am = ac;
+    ac = ap;
+    if (halo) {
+      const double hp = e(K + 1, oh);
+      s[0][hy][hx] = fma(3.0, hc, hm);
+      s[1][hy][hx] = fma(3.0, hc, hp);
+      hm = hc;
+      hc = hp;
+    }
+    __syncthreads();
+    if (I >= nc || J >= nc) continue;
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) {
+      double c[3][3];
+#pragma unroll
+      for (int y = 0; y < 3; ++y)
+#pragma unroll
+        for (int x = 0; x < 3; ++x) c[y][x] = s[kk][ty + y][tx + x];
+#pragma unroll
+      for (int jj = 0; jj < 2; ++jj) {
+        double y[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) y[x] = fma(3.0, c[1][x], c[2 * jj][x]);
+        double2* const o = reinterpret_cast<double2*>(
+            u + ((int64_t)(2 * K + kk) * n + 2 * J + jj) * n + 2 * I);
+        double2 d = *o;
+        d.x = fma(1.0 / 64.0, fma(3.0, y[1], y[0]), d.x);
+        d.y = fma(1.0 / 64.0, fma(3.0, y[1], y[2]), d.y);
+        *o = d;
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -369,6 +578,8 @@ __global__ void k_coarse_solve(Lvl L, int kind, double w, int max_sweeps, double
                                double* mu, double* om, double* t1, double* t2, double* t3,
                                const double* S1, const double* S2, const double* S3,
                                const double* b) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double red[32];
   __shared__ int done;
   const int n = L.n, half = n >> 1;
@@ -446,6 +657,8 @@ __global__ void k_residual_norm2(Lvl L, const double* __restrict__ phi,
                                  const double* __restrict__ S3,
                                  const double* __restrict__ b, double* partials,
                                  double* __restrict__ lap) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double sm[32];
   const int n = L.n;
   const int64_t cells = (int64_t)n * n * n;
@@ -736,42 +949,37 @@ cudaError_t launch_source(const Lvl& L, const double* b, const double* c, double
 
 cudaError_t launch_smooth(const Lvl& L, int lin, int sweeps, double* phi, double* mu,
                           double* om, const double* S1, const double* S2,
-                          const double* S3, const double* b, cudaStream_t st) {
+                          const double* S3, const double* b, cudaStream_t st, bool pdl) {
   const int64_t work = (int64_t)(L.n / 2) * L.n * L.n;
-  for (int s = 0; s < sweeps; ++s) {
-    for (int colour = 0; colour < 2; ++colour) {
-      if (lin == PFC_NEWTON)
-        k_smooth_colour<PFC_NEWTON><<<grid_for(work), kThreads, 0, st>>>(
-            L, colour, phi, mu, om, S1, S2, S3, b);
-      else
-        k_smooth_colour<PFC_PICARD><<<grid_for(work), kThreads, 0, st>>>(
-            L, colour, phi, mu, om, S1, S2, S3, b);
-    }
-  }
-  return cudaGetLastError();
+  const int bt = block_for(work);
+  cudaError_t e = cudaSuccess;
+  for (int s = 0; s < sweeps; ++s)
+    for (int colour = 0; colour < 2 && e == cudaSuccess; ++colour)
+      e = launch_ex(pdl, lin == PFC_NEWTON ? k_smooth_colour<PFC_NEWTON> : k_smooth_colour<PFC_PICARD>,
+                    dim3(grid_for(work, bt)), dim3(bt), 0, st, L, colour, phi, mu, om, S1, S2, S3,
+                    b);
+  return e;
 }
 
 cudaError_t launch_jacobi(const Lvl& L, int lin, int sweeps, double w, double* phi,
                           double* mu, double* om, double* t1, double* t2, double* t3,
                           const double* S1, const double* S2, const double* S3,
-                          const double* b, cudaStream_t st) {
+                          const double* b, cudaStream_t st, bool pdl) {
   const int64_t cells = (int64_t)L.n * L.n * L.n;
+  const int bt = block_for(cells);
   double* src[3] = {phi, mu, om};
   double* dst[3] = {t1, t2, t3};
-  for (int s = 0; s < sweeps; ++s) {
-    if (lin == PFC_NEWTON)
-      k_jacobi64<PFC_NEWTON><<<grid_for(cells), kThreads, 0, st>>>(
-          L, w, src[0], src[1], src[2], dst[0], dst[1], dst[2], S1, S2, S3, b);
-    else
-      k_jacobi64<PFC_PICARD><<<grid_for(cells), kThreads, 0, st>>>(
-          L, w, src[0], src[1], src[2], dst[0], dst[1], dst[2], S1, S2, S3, b);
+  cudaError_t e = cudaSuccess;
+  for (int s = 0; s < sweeps && e == cudaSuccess; ++s) {
+    e = launch_ex(pdl, lin == PFC_NEWTON ? k_jacobi64<PFC_NEWTON> : k_jacobi64<PFC_PICARD>,
+                  dim3(grid_for(cells, bt)), dim3(bt), 0, st, L, w, src[0], src[1], src[2],
+                  dst[0], dst[1], dst[2], S1, S2, S3, b);
     for (int q = 0; q < 3; ++q) {
       double* x = src[q];
       src[q] = dst[q];
       dst[q] = x;
     }
   }
-  cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && (sweeps & 1)) {
     for (int q = 0; q < 3 && e == cudaSuccess; ++q)
       e = cudaMemcpyAsync(q == 0 ? phi : q == 1 ? mu : om, src[q], cells * sizeof(double),
@@ -790,75 +998,86 @@ cudaError_t launch_residual(const Lvl& L, const double* phi, const double* mu,
   return cudaGetLastError();
 }
 
+// Coarse levels of at least this size take the tiled / block-sum kernels of the
+// FP64 transfers, which save FP64 operations but run one thread per coarse cell.
+constexpr int kLargeNc = 32;
+
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
 cudaError_t launch_residual_restrict(const Lvl& L, const double* phi, const double* mu,
-                                     const double* om, const double* S1,
-                                     const double* S2, const double* S3, const double* b,
-                                     double* rc1, double* rc2, double* rc3, double* uc1,
-                                     double* uc2, double* uc3, double* wc1, double* wc2,
-                                     double* wc3, cudaStream_t st) {
+                                     const double* om, const double* S1, const double* S2,
+                                     const double* S3, const double* b, double* rc1,
+                                     double* rc2, double* rc3, double* uc1, double* uc2,
+                                     double* uc3, double* wc1, double* wc2, double* wc3,
+                                     cudaStream_t st, bool pdl) {
   const int nc = L.n / 2;
   const int64_t work = (int64_t)nc * nc * nc;
-  k_residual_restrict<<<grid_for(work), kThreads, 0, st>>>(
-      L, phi, mu, om, S1, S2, S3, b, rc1, rc2, rc3, uc1, uc2, uc3, wc1, wc2, wc3);
-  return cudaGetLastError();
+  if (nc >= kLargeNc && aligned16(phi) && aligned16(mu) && aligned16(om) && aligned16(S1) &&
+      aligned16(S2) && aligned16(S3) && aligned16(b))
+    return launch_ex(pdl, k_residual_restrict, dim3(grid_for(work, 128)), dim3(128), 0, st, L, phi,
+                     mu, om, S1, S2, S3, b, rc1, rc2, rc3, uc1, uc2, uc3, wc1, wc2, wc3);
+  const int bt = block_for(8 * work);
+  return launch_ex(pdl, k_residual_restrict8, dim3(grid_for(8 * work, bt)), dim3(bt), 0, st, L,
+                   phi, mu, om, S1, S2, S3, b, rc1, rc2, rc3, uc1, uc2, uc3, wc1, wc2, wc3);
 }
 
-cudaError_t launch_restrict(int n, const double* fine, double* coarse, cudaStream_t st) {
+cudaError_t launch_restrict(int n, const double* fine, double* coarse, cudaStream_t st, bool pdl) {
   const int nc = n / 2;
   const int64_t work = (int64_t)nc * nc * nc;
-  k_restrict<<<grid_for(work), kThreads, 0, st>>>(n, fine, coarse);
-  return cudaGetLastError();
+  const int bt = block_for(work);
+  return launch_ex(pdl, k_restrict, dim3(grid_for(work, bt)), dim3(bt), 0, st, n, fine, coarse);
 }
 
 cudaError_t launch_coarse_source(const Lvl& Lc, const double* uc1, const double* uc2,
                                  const double* uc3, const double* bc, double* r1,
-                                 double* r2, double* r3, cudaStream_t st) {
+                                 double* r2, double* r3, cudaStream_t st, bool pdl) {
   const int64_t cells = (int64_t)Lc.n * Lc.n * Lc.n;
-  k_coarse_source<<<grid_for(cells), kThreads, 0, st>>>(Lc, uc1, uc2, uc3, bc, r1, r2, r3);
-  return cudaGetLastError();
+  const int bt = block_for(cells);
+  return launch_ex(pdl, k_coarse_source, dim3(grid_for(cells, bt)), dim3(bt), 0, st, Lc, uc1, uc2,
+                   uc3, bc, r1, r2, r3);
 }
 
-cudaError_t launch_coarse_diff(int nc, const double* v1, const double* v2,
-                               const double* v3, double* w1, double* w2, double* w3,
-                               cudaStream_t st) {
-  const int64_t cells = (int64_t)nc * nc * nc;
-  k_coarse_diff<<<grid_for(cells), kThreads, 0, st>>>(cells, v1, v2, v3, w1, w2, w3);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_prolong_add(int n, const double* e1, const double* e2,
-                               const double* e3, double* u1, double* u2, double* u3,
-                               cudaStream_t st) {
+cudaError_t launch_prolong_add(int n, const double* v1, const double* v2, const double* v3,
+                               const double* w1, const double* w2, const double* w3, double* u1,
+                               double* u2, double* u3, cudaStream_t st, bool pdl) {
+  const int nc = n / 2;
+  if (nc >= kLargeNc && aligned16(u1) && aligned16(u2) && aligned16(u3)) {
+    // eight coarse planes a block where that leaves two blocks per SM
+    const int tiles = ((nc + kPfI - 1) / kPfI) * ((nc + kPfJ - 1) / kPfJ) * 3;
+    int zc = 8;
+    while (zc > 2 && (int64_t)tiles * ((nc + zc - 1) / zc) < 2 * 152) zc >>= 1;
+    const dim3 grid((nc + kPfI - 1) / kPfI, (nc + kPfJ - 1) / kPfJ, 3 * ((nc + zc - 1) / zc));
+    return launch_ex(pdl, k_prolong_add_tile, grid, dim3(kPfI * kPfJ), 0, st, n, zc, v1, v2, v3, w1,
+                     w2, w3, u1, u2, u3);
+  }
   const int64_t cells = (int64_t)n * n * n;
-  k_prolong_add<<<grid_for(cells), kThreads, 0, st>>>(n, e1, e2, e3, u1, u2, u3);
-  return cudaGetLastError();
+  const int bt = block_for(cells);
+  return launch_ex(pdl, k_prolong_add, dim3(grid_for(cells, bt), 3), dim3(bt), 0, st, n, v1, v2, v3,
+                   w1, w2, w3, u1, u2, u3);
 }
 
 cudaError_t launch_coarse_solve(const Lvl& L, int lin, int kind, double w, int max_sweeps,
                                 double* phi, double* mu, double* om, double* t1, double* t2,
                                 double* t3, const double* S1, const double* S2,
-                                const double* S3, const double* b, cudaStream_t st) {
+                                const double* S3, const double* b, cudaStream_t st, bool pdl) {
   const int work = L.n * L.n * L.n;
   int threads = ((work + 31) / 32) * 32;
   if (threads > 1024) threads = 1024;
-  if (lin == PFC_NEWTON)
-    k_coarse_solve<PFC_NEWTON><<<1, threads, 0, st>>>(L, kind, w, max_sweeps, phi, mu, om,
-                                                       t1, t2, t3, S1, S2, S3, b);
-  else
-    k_coarse_solve<PFC_PICARD><<<1, threads, 0, st>>>(L, kind, w, max_sweeps, phi, mu, om,
-                                                       t1, t2, t3, S1, S2, S3, b);
-  return cudaGetLastError();
+  return launch_ex(pdl, lin == PFC_NEWTON ? k_coarse_solve<PFC_NEWTON> : k_coarse_solve<PFC_PICARD>,
+                   dim3(1), dim3(threads), 0, st, L, kind, w, max_sweeps, phi, mu, om, t1, t2, t3,
+                   S1, S2, S3, b);
 }
 
 cudaError_t launch_residual_norm2(const Lvl& L, const double* phi, const double* mu,
                                   const double* om, const double* S1, const double* S2,
                                   const double* S3, const double* b, double* partials,
-                                  double* out, cudaStream_t st, double* lap) {
+                                  double* out, cudaStream_t st, double* lap, bool pdl,
+                                  const DecideArgs* da, bool* decided) {
   const int nb = reduce_blocks((int64_t)L.n * L.n * L.n);
-  k_residual_norm2<<<nb, kReduceThreads, 0, st>>>(L, phi, mu, om, S1, S2, S3, b, partials,
-                                                  lap);
-  k_reduce_final<1><<<1, kReduceThreads, 0, st>>>(partials, nb, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_ex(pdl, k_residual_norm2, dim3(nb), dim3(kReduceThreads), 0, st, L, phi,
+                            mu, om, S1, S2, S3, b, partials, lap);
+  if (e == cudaSuccess) e = launch_reduce1(pdl, partials, nb, out, 1, st, da, decided);
+  return e;
 }
 
 cudaError_t launch_decide(cudaGraphConditionalHandle handle, int use_handle,

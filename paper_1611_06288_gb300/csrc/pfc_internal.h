@@ -134,13 +134,13 @@ cudaError_t launch_source(const Lvl& L, const double* b, const double* c, double
                           double* S3, cudaStream_t st);
 cudaError_t launch_smooth(const Lvl& L, int lin, int sweeps, double* phi, double* mu,
                           double* om, const double* S1, const double* S2,
-                          const double* S3, const double* b, cudaStream_t st);
+                          const double* S3, const double* b, cudaStream_t st, bool pdl = false);
 // `sweeps` damped collective Jacobi sweeps ping-ponging through t1..3; the
 // result is left in phi, mu, om.
 cudaError_t launch_jacobi(const Lvl& L, int lin, int sweeps, double w, double* phi,
                           double* mu, double* om, double* t1, double* t2, double* t3,
                           const double* S1, const double* S2, const double* S3,
-                          const double* b, cudaStream_t st);
+                          const double* b, cudaStream_t st, bool pdl = false);
 cudaError_t launch_residual(const Lvl& L, const double* phi, const double* mu,
                             const double* om, const double* S1, const double* S2,
                             const double* S3, const double* b, double* r1, double* r2,
@@ -150,23 +150,21 @@ cudaError_t launch_residual_restrict(const Lvl& L, const double* phi, const doub
                                      const double* S2, const double* S3, const double* b,
                                      double* rc1, double* rc2, double* rc3, double* uc1,
                                      double* uc2, double* uc3, double* wc1, double* wc2,
-                                     double* wc3, cudaStream_t st);
-cudaError_t launch_restrict(int n, const double* fine, double* coarse, cudaStream_t st);
+                                     double* wc3, cudaStream_t st, bool pdl = false);
+cudaError_t launch_restrict(int n, const double* fine, double* coarse, cudaStream_t st,
+                            bool pdl = false);
 cudaError_t launch_coarse_source(const Lvl& Lc, const double* uc1, const double* uc2,
                                  const double* uc3, const double* bc, double* r1,
-                                 double* r2, double* r3, cudaStream_t st);
-// e_c = v_c - w_c in place over w_c (three coarse fields of size nc^3).
-cudaError_t launch_coarse_diff(int nc, const double* v1, const double* v2,
-                               const double* v3, double* w1, double* w2, double* w3,
-                               cudaStream_t st);
-// u += P e_c for a fine level of size n (e_c on n/2).
-cudaError_t launch_prolong_add(int n, const double* e1, const double* e2,
-                               const double* e3, double* u1, double* u2, double* u3,
-                               cudaStream_t st);
+                                 double* r2, double* r3, cudaStream_t st, bool pdl = false);
+// u += P (v - w) for a fine level of size n (v, w on n/2).
+cudaError_t launch_prolong_add(int n, const double* v1, const double* v2, const double* v3,
+                               const double* w1, const double* w2, const double* w3, double* u1,
+                               double* u2, double* u3, cudaStream_t st, bool pdl = false);
 cudaError_t launch_coarse_solve(const Lvl& L, int lin, int kind, double w, int max_sweeps,
                                 double* phi, double* mu, double* om, double* t1, double* t2,
                                 double* t3, const double* S1, const double* S2,
-                                const double* S3, const double* b, cudaStream_t st);
+                                const double* S3, const double* b, cudaStream_t st,
+                                bool pdl = false);
 
 // Smoother kind of a level of spacing h under the parameters' policy.
 inline int level_kind(const pfc_params* p, double h) {
@@ -180,7 +178,13 @@ inline int level_kind(const pfc_params* p, double h) {
 cudaError_t launch_residual_norm2(const Lvl& L, const double* phi, const double* mu,
                                   const double* om, const double* S1, const double* S2,
                                   const double* S3, const double* b, double* partials,
-                                  double* out, cudaStream_t st, double* lap = nullptr);
+                                  double* out, cudaStream_t st, double* lap = nullptr,
+                                  bool pdl = false, const DecideArgs* da = nullptr,
+                                  bool* decided = nullptr);
+// The final reduction of a residual's block sums, one block per member: with a
+// decision to take (single member) it is part of the same launch (*decided).
+cudaError_t launch_reduce1(bool pdl, const double* partials, int nparts, double* out, int members,
+                           cudaStream_t st, const DecideArgs* da, bool* decided);
 // Unscaled 7-point Laplacian (neighbour sum - 6 centre) of a field.
 cudaError_t launch_laplacian(int n, const double* v, double* lap, cudaStream_t st,
                              int members = 1);

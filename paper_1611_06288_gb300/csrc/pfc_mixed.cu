@@ -1137,20 +1137,6 @@ __global__ void k_reduce1_decide(const double* __restrict__ partials, int nparts
   }
 }
 
-// The final reduction of a residual's block sums: with a decision to take
-// (single member) the fused kernel, else k_reduce1.
-cudaError_t launch_reduce1(bool pdl, const double* partials, int nparts, double* out,
-                           int members, cudaStream_t st, const DecideArgs* da, bool* decided) {
-  if (da && members == 1) {
-    if (decided) *decided = true;
-    return launch_ex(pdl, k_reduce1_decide, dim3(1), dim3(kReduceThreads), 0, st, partials,
-                     nparts, out, *da);
-  }
-  if (decided) *decided = false;
-  return launch_ex(pdl, k_reduce1, dim3(members), dim3(kReduceThreads), 0, st, partials, nparts,
-                   out);
-}
-
 // 8-cell average of a split-layout field onto the (split-layout) level n/2.
 __global__ void k_restrict32(int n, const float* __restrict__ f, float* __restrict__ c) {
   pdl_wait();
@@ -3887,6 +3873,18 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
 }
 
 }  // namespace
+
+cudaError_t launch_reduce1(bool pdl, const double* partials, int nparts, double* out,
+                           int members, cudaStream_t st, const DecideArgs* da, bool* decided) {
+  if (da && members == 1) {
+    if (decided) *decided = true;
+    return launch_ex(pdl, k_reduce1_decide, dim3(1), dim3(kReduceThreads), 0, st, partials,
+                     nparts, out, *da);
+  }
+  if (decided) *decided = false;
+  return launch_ex(pdl, k_reduce1, dim3(members), dim3(kReduceThreads), 0, st, partials, nparts,
+                   out);
+}
 
 // Planes per block of k_defect64_fx: the split of the n planes of a column
 // into chunks that minimises the waves of resident blocks times the planes
