@@ -21,6 +21,7 @@ struct Lvl {
   double gh;    // 1/(2 h^2)
   double Q0;    // 18/h^4      (the 6/h^2 * 3/h^2 coupling of rows 2 and 3)
   double c1;    // (1 - eps)/2
+  double cQ;    // c1 + Q0
 };
 
 inline Lvl make_lvl(int n, double h, double eps, double tau) {
@@ -35,6 +36,7 @@ inline Lvl make_lvl(int n, double h, double eps, double tau) {
   L.gh = 0.5 * g;
   L.Q0 = 18.0 * g * g;
   L.c1 = 0.5 * (1.0 - eps);
+  L.cQ = L.c1 + L.Q0;
   return L;
 }
 
@@ -73,45 +75,9 @@ __device__ __forceinline__ T nbsum_coherent(const T* v, const Stencil& s) {
   return ((v[s.xm] + v[s.xp]) + (v[s.ym] + v[s.yp])) + (v[s.zm] + v[s.zp]);
 }
 
-// Cubic term f(a) = (a+b)(a^2+b^2)/4 of Eq. 5.2 and its derivative in a.
+// Cubic term f(a) = (a+b)(a^2+b^2)/4 of Eq. 5.2.
 __device__ __forceinline__ double cubic_f(double a, double b) {
   return 0.25 * (a + b) * fma(a, a, b * b);
-}
-__device__ __forceinline__ double cubic_fp(double a, double b) {
-  return fma(0.75 * a, a, fma(0.5 * a, b, 0.25 * b * b));
-}
-
-// Pointwise solve of the smoother's 3x3 system (Section 5)
-//   [ 1      kap   0   ] [phi]   [st1 = S1 + tau/h^2 sum mu_nb   ]
-//   [ -q     1     6g  ] [mu ] = [st2 = S2 + extra + g sum om_nb ]
-//   [ 3g     0     1   ] [om ]   [st3 = S3 + g/2 sum phi_nb      ]
-// by eliminating phi and om: mu = (st2 - 6g st3 + (q + 18 g^2) st1) / det,
-// det = 1 + kap (q + 18 g^2) >= 1 because q > 0.  The Newton variant uses
-// q = f'(phi_n) + (1-eps)/2, extra = f(phi_n) - f'(phi_n) phi_n; the paper's
-// Picard variant q = (phi_n^2 + b^2)/4 + (1-eps)/2, extra = (phi_n^2+b^2) b/4.
-template <int LIN>
-__device__ __forceinline__ void point_solve(const Lvl& L, double sphi, double smu,
-                                            double som, double phin, double b,
-                                            double s1, double s2, double s3,
-                                            double& phi, double& mu, double& om) {
-  const double st1 = fma(L.tg, smu, s1);
-  const double st3 = fma(L.gh, sphi, s3);
-  double q, extra;
-  if (LIN == PFC_NEWTON) {
-    const double fp = cubic_fp(phin, b);
-    q = fp + L.c1;
-    extra = fma(-fp, phin, cubic_f(phin, b));
-  } else {
-    const double p = 0.25 * fma(phin, phin, b * b);
-    q = p + L.c1;
-    extra = p * b;
-  }
-  const double st2 = fma(L.g, som, s2 + extra);
-  const double Q = q + L.Q0;
-  const double det = fma(L.kap, Q, 1.0);
-  mu = fma(Q, st1, fma(-L.g6, st3, st2)) / det;
-  phi = fma(-L.kap, mu, st1);
-  om = fma(-L.g3, phi, st3);
 }
 
 // r = S - N(u) at one cell (Eqs. 5.4-5.6 with M = 1); lap receives the
@@ -237,6 +203,65 @@ __device__ __forceinline__ double f2d(float f) {
   if (e - 1u > 253u) return f2d_special(u);             // e == 0 or e == 255
   const unsigned hi = (u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xFFFFFu);
   return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// 1/x within 1 ulp for a normal x, without the scaling of subnormal divisors
+// that __fdividef carries: num * rcp_approx(det) equals __fdividef(num, det)
+// for the determinants of the pointwise solve, which are >= 1.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// a / d for d >= 1 in 5 FP64 operations (a division is about 10, and the FP64
+// pipe is what bounds the smoother): the FP32 reciprocal of d, one Newton step
+// r (2 - d r) to about 2^-46, and the quotient a r corrected by its exact
+// remainder a - d q, which leaves the rounding of the last operation.  Beyond
+// FP32's range (or NaN) the division itself.
+__device__ __forceinline__ double div_by(double a, double d) {
+  const float df = d2f_rn(d);
+  if (!(df < 1e37f)) return a / d;
+  double r = f2d(rcp_approx(df));
+  r = fma(r, fma(-d, r, 1.0), r);
+  const double q = a * r;
+  return fma(r, fma(-d, q, a), q);
+}
+
+// Pointwise solve of the smoother's 3x3 system (Section 5)
+//   [ 1      kap   0   ] [phi]   [st1 = S1 + tau/h^2 sum mu_nb   ]
+//   [ -q     1     6g  ] [mu ] = [st2 = S2 + extra + g sum om_nb ]
+//   [ 3g     0     1   ] [om ]   [st3 = S3 + g/2 sum phi_nb      ]
+// by eliminating phi and om: mu = (st2 - 6g st3 + (q + 18 g^2) st1) / det,
+// det = 1 + kap (q + 18 g^2) >= 1 because q > 0.  The Newton variant uses
+// q = f'(phi_n) + (1-eps)/2, extra = f(phi_n) - f'(phi_n) phi_n; the paper's
+// Picard variant q = (phi_n^2 + b^2)/4 + (1-eps)/2, extra = (phi_n^2+b^2) b/4.
+// With f = (a+b)(a^2+b^2)/4: f' = (2 a^2 + (a+b)^2)/4 and f - f' a = (b^3 -
+// a^2 (2a + b))/4, 23 FP64 operations with the quotient (33 before; a colour
+// pass of 128^3 92 -> 77 us).
+template <int LIN>
+__device__ __forceinline__ void point_solve(const Lvl& L, double sphi, double smu,
+                                            double som, double phin, double b,
+                                            double s1, double s2, double s3,
+                                            double& phi, double& mu, double& om) {
+  const double st1 = fma(L.tg, smu, s1);
+  const double st3 = fma(L.gh, sphi, s3);
+  const double a2 = phin * phin, b2 = b * b;
+  double q4, extra4;                       // 4 (q - c1), 4 extra
+  if (LIN == PFC_NEWTON) {
+    const double s = phin + b;
+    q4 = fma(2.0, a2, s * s);
+    extra4 = fma(-a2, fma(2.0, phin, b), b2 * b);
+  } else {
+    q4 = a2 + b2;
+    extra4 = q4 * b;
+  }
+  const double st2 = fma(L.g, som, fma(0.25, extra4, s2));
+  const double Q = fma(0.25, q4, L.cQ);
+  const double det = fma(L.kap, Q, 1.0);
+  mu = div_by(fma(Q, st1, fma(-L.g6, st3, st2)), det);
+  phi = fma(-L.kap, mu, st1);
+  om = fma(-L.g3, phi, st3);
 }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream

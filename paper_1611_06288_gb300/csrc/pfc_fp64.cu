@@ -240,7 +240,8 @@ __global__ void k_residual(Lvl L, const double* __restrict__ phi,
 //
 // Small grids: eight lanes per coarse cell, one child each, summed by the
 // first lane in the children's order.  (One thread per coarse cell ran the
-// eight residuals one after another: 24 us at every size up to 32^3.)
+// eight residuals one after another: 24 us at every size up to 32^3, now 6 to
+// 9 us.)
 // ---------------------------------------------------------------------------
 __global__ void k_residual_restrict8(Lvl L, const double* __restrict__ phi,
                                      const double* __restrict__ mu,
@@ -335,7 +336,7 @@ struct BlockAt {
 // children are summed as sum_out - 3 sum_in (the inner faces of the block
 // cancel) and the linear terms of the rows from the sums, which takes 21
 // instead of 40 FP64 operations per fine cell: the pass is bound by the FP64
-// pipe (128^3: 154 -> 87 us).  n even, pointers 16-byte aligned.
+// pipe (128^3: 154 -> 90 us).  n even, pointers 16-byte aligned.
 __global__ void __launch_bounds__(128) k_residual_restrict(
     Lvl L, const double* __restrict__ phi, const double* __restrict__ mu,
     const double* __restrict__ om, const double* __restrict__ S1, const double* __restrict__ S2,
@@ -475,7 +476,7 @@ __global__ void k_prolong_add(int n, const double* __restrict__ v1, const double
 // Large levels: the interpolation as one-dimensional passes, z then y then x
 // ((3 e_0 + e_-1) / 4 and (3 e_0 + e_+1) / 4 per axis), 31 FP64 operations per
 // eight children and component instead of 64: the pass is bound by the FP64
-// pipe (128^3: 99 -> 44 us).  A block of kPfI x kPfJ threads owns that tile of
+// pipe (128^3: 99 -> 68 us).  A block of kPfI x kPfJ threads owns that tile of
 // coarse columns of one component and marches over zc coarse planes; each
 // thread interpolates its own column (and at most one of the tile's halo) in z
 // from values it carries, the tile's columns meet in shared memory (double
@@ -567,25 +568,44 @@ __global__ void __launch_bounds__(kPfI * kPfJ) k_prolong_add_tile(
 }
 
 // ---------------------------------------------------------------------------
-// a5: coarsest level: sweeps in one thread block until the largest relative
+// a5: coarsest level: sweeps in one thread block until every value's relative
 // change falls below 1e-14 or max_sweeps.  Red-black (kind 0) updates in
 // place; damped Jacobi (kind 1) computes every cell into t and copies back.
-// Neighbours are read with coherent loads because this block wrote them in
-// the previous half-sweep.
+// Levels of at most kCoarseSmem cells a side run in shared memory (`shared`);
+// a larger one reads neighbours with coherent loads because this block wrote
+// them in the previous half-sweep.  The test |x - x_old| < 1e-14 (1 + |x|) is
+// a comparison and a block vote: as a division and a maximum per value it was
+// a third of a sweep's FP64 operations.
 // ---------------------------------------------------------------------------
+constexpr int kCoarseSmem = 8;
+
+__device__ __forceinline__ bool settled(double x, double old) {
+  return !(fabs(x - old) >= 1e-14 * (1.0 + fabs(x)));     // true for NaN: ends the sweeps
+}
+
 template <int LIN>
-__global__ void k_coarse_solve(Lvl L, int kind, double w, int max_sweeps, double* phi,
-                               double* mu, double* om, double* t1, double* t2, double* t3,
-                               const double* S1, const double* S2, const double* S3,
+__global__ void k_coarse_solve(Lvl L, int kind, double w, int max_sweeps, int shared,
+                               double* gphi, double* gmu, double* gom, double* t1, double* t2,
+                               double* t3, const double* S1, const double* S2, const double* S3,
                                const double* b) {
   pdl_wait();
   pdl_trigger();
-  __shared__ double red[32];
-  __shared__ int done;
+  extern __shared__ double cs[];
   const int n = L.n, half = n >> 1;
   const int ncell = n * n * n;
+  double *phi = gphi, *mu = gmu, *om = gom;
+  if (shared) {
+    const double* const from[7] = {gphi, gmu, gom, S1, S2, S3, b};
+#pragma unroll
+    for (int f = 0; f < 7; ++f)
+      for (int t = threadIdx.x; t < ncell; t += blockDim.x) cs[f * ncell + t] = from[f][t];
+    phi = cs, mu = cs + ncell, om = cs + 2 * ncell;
+    S1 = cs + 3 * ncell, S2 = cs + 4 * ncell, S3 = cs + 5 * ncell, b = cs + 6 * ncell;
+    t1 = cs + 7 * ncell, t2 = cs + 8 * ncell, t3 = cs + 9 * ncell;
+    __syncthreads();
+  }
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    double change = 0.0;
+    bool done = true;
     if (kind == PFC_SWEEP_JACOBI) {
       for (int t = threadIdx.x; t < ncell; t += blockDim.x) {
         const int i = t % n, j = (t / n) % n, k = t / (n * n);
@@ -601,17 +621,15 @@ __global__ void k_coarse_solve(Lvl L, int kind, double w, int max_sweeps, double
       }
       __syncthreads();
       for (int t = threadIdx.x; t < ncell; t += blockDim.x) {
-        change = fmax(change, fabs(t1[t] - phi[t]) / (1.0 + fabs(t1[t])));
-        change = fmax(change, fabs(t2[t] - mu[t]) / (1.0 + fabs(t2[t])));
-        change = fmax(change, fabs(t3[t] - om[t]) / (1.0 + fabs(t3[t])));
+        done = done && settled(t1[t], phi[t]) && settled(t2[t], mu[t]) && settled(t3[t], om[t]);
         phi[t] = t1[t];
         mu[t] = t2[t];
         om[t] = t3[t];
       }
-      __syncthreads();
     } else {
       const int cells = half * n * n;
       for (int colour = 0; colour < 2; ++colour) {
+        if (colour) __syncthreads();
         for (int t = threadIdx.x; t < cells; t += blockDim.x) {
           const int p = t % half, r = t / half;
           const int j = r % n, k = r / n;
@@ -625,25 +643,18 @@ __global__ void k_coarse_solve(Lvl L, int kind, double w, int max_sweeps, double
           phi[s.c] = np;
           mu[s.c] = nm;
           om[s.c] = nw;
-          change = fmax(change, fabs(np - op) / (1.0 + fabs(np)));
-          change = fmax(change, fabs(nm - om_) / (1.0 + fabs(nm)));
-          change = fmax(change, fabs(nw - ow) / (1.0 + fabs(nw)));
+          done = done && settled(np, op) && settled(nm, om_) && settled(nw, ow);
         }
-        __syncthreads();
       }
     }
-    // block max of the change
-    for (int o = 16; o > 0; o >>= 1) change = fmax(change, __shfl_down_sync(0xffffffffu, change, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = change;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double m = 0.0;
-      for (int q = 0; q < (int)((blockDim.x + 31) >> 5); ++q) m = fmax(m, red[q]);
-      done = (m < 1e-14);
-    }
-    __syncthreads();
-    if (done) break;
+    if (__syncthreads_and(done)) break;
   }
+  if (shared)
+    for (int t = threadIdx.x; t < ncell; t += blockDim.x) {
+      gphi[t] = phi[t];
+      gmu[t] = mu[t];
+      gom[t] = om[t];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1063,9 +1074,11 @@ cudaError_t launch_coarse_solve(const Lvl& L, int lin, int kind, double w, int m
   const int work = L.n * L.n * L.n;
   int threads = ((work + 31) / 32) * 32;
   if (threads > 1024) threads = 1024;
+  const int shared = L.n <= kCoarseSmem;
+  const size_t smem = shared ? (size_t)10 * work * sizeof(double) : 0;   // <= 40 KiB
   return launch_ex(pdl, lin == PFC_NEWTON ? k_coarse_solve<PFC_NEWTON> : k_coarse_solve<PFC_PICARD>,
-                   dim3(1), dim3(threads), 0, st, L, kind, w, max_sweeps, phi, mu, om, t1, t2, t3,
-                   S1, S2, S3, b);
+                   dim3(1), dim3(threads), smem, st, L, kind, w, max_sweeps, shared, phi, mu, om,
+                   t1, t2, t3, S1, S2, S3, b);
 }
 
 cudaError_t launch_residual_norm2(const Lvl& L, const double* phi, const double* mu,

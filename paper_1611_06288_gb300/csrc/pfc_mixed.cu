@@ -1155,15 +1155,6 @@ __global__ void k_restrict32(int n, const float* __restrict__ f, float* __restri
   c[split_index(I, J, K, nc)] = 0.125f * acc;
 }
 
-// 1/x within 1 ulp for a normal x, without the scaling of subnormal divisors
-// that __fdividef carries: num * rcp_approx(det) equals __fdividef(num, det)
-// for the determinants of the pointwise solve, which are >= 1.
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 // Pointwise solve of the linearised 3x3 system (q frozen):
 //   [ 1   kap  0  ] [dp]   [r1 + tau/h^2 sum d_mu]
 //   [ -q  1    6g ] [dm] = [r2 + g sum d_om      ]
