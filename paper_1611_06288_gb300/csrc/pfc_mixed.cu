@@ -2801,92 +2801,20 @@ __device__ void tail_vcycle(float* smem, const TailParams& P, bool zero_top, flo
   }
 }
 
-// The whole tail lives in shared memory.  The top level's r and q (and d
-// when it does not start from zero) are loaded from global memory, the lower
-// levels' q are restricted in shared memory, and the top level's d is stored
-// back at the end.
-__global__ void __launch_bounds__(kTailThreads) k_lin_tail32(TailParams P) {
-  pdl_wait();
-  pdl_trigger();
-  extern __shared__ float smem[];
-  __shared__ float red[2][32];
-  __shared__ int done;
-  const bool zero_top = P.zero_init != 0;
-  // one block per member of a batched launch; P itself stays unmodified (a
-  // written parameter struct would be copied to local memory)
-  const size_t off = (size_t)blockIdx.x * P.L[0].n * P.L[0].n * P.L[0].n;
-  float* const gd0 = P.gd[0] + off;
-  float* const gd1 = P.gd[1] + off;
-  float* const gd2 = P.gd[2] + off;
-  {
-    const float* const gr0 = P.gr[0] + off;
-    const float* const gr1 = P.gr[1] + off;
-    const float* const gr2 = P.gr[2] + off;
-    const float* const gq = P.gq + off;
-    const SLev S0 = slev(smem, P, 0);
-    const int n0 = P.L[0].n;
-    const int cells = n0 * n0 * n0;
-    // all of a thread's global loads of a batch before any shared-memory
-    // store: one memory round trip per batch instead of one per value
-    constexpr int kB = 4;
-    for (int t0 = threadIdx.x; t0 < cells; t0 += kB * blockDim.x) {
-      float v[7][kB];
-#pragma unroll
-      for (int u = 0; u < kB; ++u) {
-        const int t = t0 + u * blockDim.x;
-        if (t < cells) {
-          v[0][u] = gr0[t];
-          v[1][u] = gr1[t];
-          v[2][u] = gr2[t];
-          v[3][u] = gq[t];
-          if (!zero_top) {
-            v[4][u] = gd0[t];
-            v[5][u] = gd1[t];
-            v[6][u] = gd2[t];
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kB; ++u) {
-        const int t = t0 + u * blockDim.x;
-        if (t < cells) {
-          int p, j, k, colour;
-          split_cell(t, n0, p, j, k, colour);
-          const int o = (2 * p + ((j + k + colour) & 1)) + n0 * (j + n0 * k);   // natural index
-          S0.r0[o] = v[0][u];
-          S0.r1[o] = v[1][u];
-          S0.r2[o] = v[2][u];
-          S0.q[o] = v[3][u];
-          if (!zero_top) {
-            S0.d0[o] = v[4][u];
-            S0.d1[o] = v[5][u];
-            S0.d2[o] = v[6][u];
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  tail_qrestrict(smem, P);
-  tail_vcycle(smem, P, zero_top, red, &done);
-  const SLev S0 = slev(smem, P, 0);
-  const int n0 = P.L[0].n;
-  const int cells = n0 * n0 * n0;
-  for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-    int p, j, k, colour;
-    split_cell(t, n0, p, j, k, colour);
-    const int o = (2 * p + ((j + k + colour) & 1)) + n0 * (j + n0 * k);
-    gd0[t] = S0.d0[o];
-    gd1[t] = S0.d1[o];
-    gd2[t] = S0.d2[o];
-  }
+#include "pfc_tail.cuh"
+
+// Shared memory of the tail starting at level l0.
+size_t tail_smem_bytes(const int* sizes, int l0, int nl) {
+  size_t floats = 0;
+  for (int l = l0; l < nl; ++l) floats += tail_floats(sizes[l]);
+  return floats * sizeof(float);
 }
 
-// Shared memory of the tail starting at level l0 (10 floats per cell per level).
-size_t tail_smem_bytes(const int* sizes, int l0, int nl) {
-  size_t cells = 0;
-  for (int l = l0; l < nl; ++l) cells += (size_t)sizes[l] * sizes[l] * sizes[l];
-  return cells * 10 * sizeof(float);
+// Threads of a tail whose top level has n^3 cells: one per position (cell of
+// each colour), at most two positions a thread.
+int tail_threads(int n) {
+  const int t = (n * n * n / 2 + 31) / 32 * 32;
+  return t < 64 ? 64 : t > kTailThreads ? kTailThreads : t;
 }
 
 constexpr size_t kTailMaxSmem = 200 * 1024;   // + static shared memory <= 227 KiB
@@ -3629,7 +3557,7 @@ cudaError_t tail32(const Ctx32& c, int l0, bool zero_init) {
   }
   prof_begin(c.pr, PFC_K_LIN_COARSE, c.st);
   cudaError_t e =
-      launch_k(c.pr == nullptr, k_lin_tail32, dim3(c.nb), dim3(kTailThreads), smem, c.st, P);
+      launch_k(c.pr == nullptr, k_lin_tail32, dim3(c.nb), dim3(tail_threads(sizes[l0])), smem, c.st, P);
   prof_end(c.pr, PFC_K_LIN_COARSE, l0, 1, c.st);
   return e;
 }
@@ -3745,16 +3673,19 @@ cudaError_t ctail32(const Ctx32& c, int l0, bool zero_init, int nd, size_t smem,
   return e;
 }
 
+// Whether the single-block tail takes the levels from l on (where the cluster
+// tail does not).
+bool block_tail_at(const Ctx32& c, int l) {
+  if (c.L[l].n > kTailMaxN || c.nl - l > kTailMaxLevels) return false;
+  int sizes[kMaxLevelsMixed];
+  for (int q = 0; q < c.nl; ++q) sizes[q] = c.L[q].n;
+  return tail_smem_bytes(sizes, l, c.nl) <= kTailMaxSmem;
+}
+
 // Whether vcycle32 at level l restricts to l + 1 with a launch of its own
 // (not the cluster tail, the shared-memory tail or the coarsest solve).
 bool restricts_alone(const Ctx32& c, int l) {
-  if (c.p->cluster_tail == 1 || l >= c.nl - 1) return false;
-  if (c.L[l].n <= kTailMaxN && c.nl - l <= kTailMaxLevels) {
-    int sizes[kMaxLevelsMixed];
-    for (int q = 0; q < c.nl; ++q) sizes[q] = c.L[q].n;
-    if (tail_smem_bytes(sizes, l, c.nl) <= kTailMaxSmem) return false;
-  }
-  return true;
+  return c.p->cluster_tail != 1 && l < c.nl - 1 && !block_tail_at(c, l);
 }
 
 // Levels below l + 1 whose restriction one k_lin_restrict_chain32 launch at
@@ -3786,11 +3717,7 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
     const int nd = ctail_layout(c, l, &smem, &ga_off);
     if (nd > 0 && ctail_supported()) return ctail32(c, l, zero_init, nd, smem, ga_off);
   }
-  if (L.n <= kTailMaxN && c.nl - l <= kTailMaxLevels) {
-    int sizes[kMaxLevelsMixed];
-    for (int q = 0; q < c.nl; ++q) sizes[q] = c.L[q].n;
-    if (tail_smem_bytes(sizes, l, c.nl) <= kTailMaxSmem) return tail32(c, l, zero_init);
-  }
+  if (block_tail_at(c, l)) return tail32(c, l, zero_init);
   if (l == c.nl - 1) {
     const int work = L.n * L.n * L.n;
     int threads = ((work + 31) / 32) * 32;
@@ -4407,10 +4334,14 @@ cudaError_t mixed_vcycles(MixedBufs& mx, const pfc_params& p, int nl, const int*
     h *= 2.0;
   }
   cudaError_t e = cudaSuccess;
-  for (int l = 1; l < nl && e == cudaSuccess;) {
+  // levels below the top one of the single-block tail take their q there
+  int nq = nl;
+  for (int l = 0; l < nl && nq == nl; ++l)
+    if (c.p->cluster_tail == 0 && block_tail_at(c, l)) nq = l + 1;
+  for (int l = 1; l < nq && e == cudaSuccess;) {
     const int nc = sizes[l];
     // up to two more levels in the same launch where the block tiles the level
-    int extra = nl - 1 - l;
+    int extra = nq - 1 - l;
     if (extra > 2) extra = 2;
     if (nc % kChTX != 0 || nc % kChTZ != 0 || nc % kChTY != 0) extra = 0;
     prof_begin(pr, PFC_K_RESTRICT, st);
