@@ -67,23 +67,19 @@ PFC_HD int fix_clz64(uint64_t a) {   // a != 0
 
 // X = round(v 2^kFixFrac), halves rounded away from zero (a symmetric
 // rounding); ok is cleared when |v| >= 2^kFixIntBits or v is not finite.
-// v = m 2^(e - 1075) with m the 53-bit significand and e the biased exponent,
-// so X = m 2^(e - 1075 + kFixFrac): a left shift by s = e - 1021 >= 0, else a
-// rounded right shift by -s (zero and subnormal inputs shift out to 0).
+// v = m 2^(e - 1075) with m the 53-bit significand and e the biased exponent;
+// with m left-justified to 64 bits, X = m 2^-(s + 1), s = 1085 - kFixFrac - e: a
+// right shift by s, then a rounded one by 1 (s > 63 shifts out to 0, also zeros
+// and subnormals; out of range, the value is not used).
 PFC_HD int64_t fix_of(double v, bool& ok) {
   const uint64_t u = fix_bits_of(v);
   const unsigned e = (unsigned)(u >> 52) & 0x7FFu;
   ok = ok && e <= kFixMaxBiasedExp;
-  const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int s = (int)e - (1075 - kFixFrac);
-  uint64_t a;
-  if (s >= 0) {
-    a = m << (s & 7);                      // s <= kFixIntBits + 1 inside the range
-  } else {
-    const int r = -s;
-    a = r < 60 ? (m + (1ull << (r - 1))) >> r : 0ull;
-  }
-  return (u >> 63) ? -(int64_t)a : (int64_t)a;
+  const uint64_t m = (u << 11) | (1ull << 63);
+  const unsigned s = 1085u - kFixFrac - e;
+  const uint64_t a = s > 63u ? 0ull : ((m >> s) + 1ull) >> 1;
+  const int64_t neg = (int64_t)u >> 63;
+  return ((int64_t)a ^ neg) - neg;
 }
 
 // X 2^-kFixFrac rounded to binary64, to nearest with ties to even.  The top
