@@ -2438,6 +2438,8 @@ struct TailParams {
   float w;
   LvlF L[kTailMaxLevels];
   int kind[kTailMaxLevels];
+  int off[kTailMaxLevels];    // of a level's fields in shared memory (k_lin_tail32)
+  int rn[kTailMaxLevels], rhalf[kTailMaxLevels];   // 65536 / n + 1, 65536 / (n / 2) + 1
   float* gd[3];      // top level in global memory
   const float* gr[3];
   const float* gq;
@@ -3536,9 +3538,15 @@ cudaError_t tail32(const Ctx32& c, int l0, bool zero_init) {
   P.coarse_sweeps = c.p->coarse_sweeps;
   P.zero_init = zero_init ? 1 : 0;
   P.w = c.w;
+  int off = 0;
   for (int l = l0; l < c.nl; ++l) {
+    const int n = c.L[l].n;
     P.L[l - l0] = c.L[l];
     P.kind[l - l0] = c.kind[l];
+    P.off[l - l0] = off;
+    P.rn[l - l0] = 65536 / n + 1;
+    P.rhalf[l - l0] = 65536 / (n / 2) + 1;
+    off += tail_floats(n);
   }
   for (int q = 0; q < 3; ++q) {
     P.gd[q] = mx.d[l0][q];

@@ -10,14 +10,14 @@
 // were bank conflicts), a thread's positions and their neighbours are the same
 // indices for both colours and are worked out once per call, and r, q of a
 // thread's cells stay in registers over the sweeps of a call.  Measured (ncu):
-// V(2,2) on 16^3 with four coarsest sweeps on 8^3 36.4 -> 23.1 us (a colour pass
-// of 16^3 takes 0.8 us, 0.65 at the shared-memory rate), 12^3 alone with two
-// sweeps 9.7 -> 7.3.
+// V(2,2) on 16^3 with four coarsest sweeps on 8^3 36.4 -> 19.6 us (a colour pass
+// of 16^3 takes 0.85 us, 0.65 at the shared-memory rate), 16^3 alone with two
+// sweeps 16.4 -> 8.3.
 
 extern __shared__ float tsm[];
 
 // A level in shared memory: component f of d, r, t, colour c, at element
-// x + (2 f + c) cs of tsm; q likewise.  cs = n^3 / 2 + n / 2: the pad puts the two
+// x + (2 f + c) cs of tsm; q likewise.  cs = n^3 / 2 + 16: the pad puts the two
 // colours of a row in different banks for the prolongation, which reads both.
 // Offsets, not pointers: a call that takes a pointer loses that it is shared
 // memory.
@@ -26,20 +26,25 @@ struct TLev {
   int hc, cs;                            // cells of a colour, distance of the colours
 };
 
-__host__ __device__ inline int tail_floats(int n) { return 10 * (n * n * n + n); }
+__host__ __device__ inline int tail_floats(int n) { return 10 * (n * n * n + 32); }
 
 __device__ __forceinline__ TLev tlev(const TailParams& P, int l) {
-  int off = 0;
-  for (int m = 0; m < l; ++m) off += tail_floats(P.L[m].n);
   const int n = P.L[l].n;
   TLev S;
   S.hc = n * n * n >> 1;
-  S.cs = S.hc + (n >> 1);
-  S.d = off;
+  S.cs = S.hc + 16;
+  S.d = P.off[l];
   S.r = S.d + 6 * S.cs;
   S.q = S.d + 12 * S.cs;
   S.t = S.d + 14 * S.cs;
   return S;
+}
+
+// x / d for x d < 2^16 from recip = 65536 / d + 1 (worked out on the host): a
+// division by a run-time number takes about 25 instructions, in phases that
+// have 100.
+__device__ __forceinline__ int small_div(int x, int recip) {
+  return (x * recip) >> 16;
 }
 
 // Position `pos` = p + half (j + n k) of both colours: the positions of its y
@@ -51,10 +56,11 @@ template <bool PAIR>
 struct TPos {
   int c, ym, yp, zm, zp, xl, xr;
   bool sg, on;
-  __device__ __forceinline__ TPos(int n, int pos) {
+  __device__ __forceinline__ TPos(const TailParams& P, int l, int pos) {
     constexpr int w = PAIR ? 2 : 1;
-    const int half = n >> 1, hp = half * n;
-    const int r = pos / half, p = pos - r * half, k = r / n, j = r - k * n;
+    const int n = P.L[l].n, half = n >> 1, hp = half * n;
+    const int r = small_div(pos, P.rhalf[l]), p = pos - r * half;
+    const int k = small_div(r, P.rn[l]), j = r - k * n;
     on = k < n;
     c = pos;
     ym = pos + (j == 0 ? hp - half : -half);
@@ -115,14 +121,17 @@ struct TVal<true> {
 // of the largest value, tested every fourth sweep (the outer FP64 loop absorbs
 // the rest).
 template <bool PAIR, int SLOTS>
-__device__ __forceinline__ void tail_sweeps(const LvlF& L, int kind, const TLev S, int sweeps,
-                                            float w, bool zero, bool coarsest, float (*red)[32],
+__device__ __forceinline__ void tail_sweeps(const TailParams& P, int l, const TLev S, int sweeps,
+                                            bool zero, bool coarsest, float (*red)[32],
                                             int* done) {
+  const LvlF L = P.L[l];
+  const int kind = P.kind[l];
+  const float w = P.w;
   using V = TVal<PAIR>;
   using T = typename V::T;
   const int cs = S.cs, step = PAIR ? 2 : 1;
-  const TPos<PAIR> pos[2] = {TPos<PAIR>(L.n, threadIdx.x * step),
-                             TPos<PAIR>(L.n, (threadIdx.x + blockDim.x) * step)};
+  const TPos<PAIR> pos[2] = {TPos<PAIR>(P, l, threadIdx.x * step),
+                             TPos<PAIR>(P, l, (threadIdx.x + blockDim.x) * step)};
   T rq[SLOTS][2][4];
 #pragma unroll
   for (int s = 0; s < SLOTS; ++s)
@@ -135,6 +144,7 @@ __device__ __forceinline__ void tail_sweeps(const LvlF& L, int kind, const TLev 
   int d = S.d, o = S.t;                  // Jacobi: d -> o, then exchanged
   for (int sweep = 0; sweep < sweeps; ++sweep) {
     const bool fresh = zero && sweep == 0;
+    const bool test = coarsest && (sweep & 3) == 3 && sweep + 1 < sweeps;
     float change = 0.f, size = 0.f;
     if (kind == PFC_SWEEP_JACOBI) {
 #pragma unroll
@@ -156,7 +166,7 @@ __device__ __forceinline__ void tail_sweeps(const LvlF& L, int kind, const TLev 
           for (int f = 0; f < 3; ++f) {
             const T v = V::step(w, x[f], old[f]);
             V::st(o + (2 * f + c) * cs + pos[s].c, v);
-            if (coarsest) {
+            if (test) {
               change = fmaxf(change, V::top(V::diff(v, old[f])));
               size = fmaxf(size, V::top(v));
             }
@@ -183,7 +193,7 @@ __device__ __forceinline__ void tail_sweeps(const LvlF& L, int kind, const TLev 
 #pragma unroll
           for (int f = 0; f < 3; ++f) {
             const int at = d + (2 * f + c) * cs + pos[s].c;
-            if (coarsest) {
+            if (test) {
               const T old = fresh ? V::all(0.f) : V::ld(at);
               change = fmaxf(change, V::top(V::diff(x[f], old)));
               size = fmaxf(size, V::top(x[f]));
@@ -194,7 +204,7 @@ __device__ __forceinline__ void tail_sweeps(const LvlF& L, int kind, const TLev 
         __syncthreads();
       }
     }
-    if (!coarsest || (sweep & 3) != 3 || sweep + 1 == sweeps) continue;
+    if (!test) continue;
     for (int b = 16; b > 0; b >>= 1) {
       change = fmaxf(change, __shfl_down_sync(0xffffffffu, change, b));
       size = fmaxf(size, __shfl_down_sync(0xffffffffu, size, b));
@@ -231,12 +241,13 @@ __device__ __forceinline__ void tail_sweeps(const LvlF& L, int kind, const TLev 
 struct TCoarse {
   int t, jj, I, J, K;
   bool on;
-  __device__ __forceinline__ TCoarse(int nc) {
-    int r = threadIdx.x / nc;                // 2 nc^3 <= blockDim (tail_threads)
+  // rnc: small_div's reciprocal of nc
+  __device__ __forceinline__ TCoarse(int nc, int rnc) {
+    int r = small_div(threadIdx.x, rnc);     // 2 nc^3 <= blockDim (tail_threads)
     I = threadIdx.x - r * nc;
     jj = r & 1;
     r >>= 1;
-    K = r / nc;
+    K = small_div(r, rnc);
     J = r - K * nc;
     on = K < nc;
     t = I + nc * r;
@@ -249,10 +260,11 @@ struct TCoarse {
 // rho = r - J d of the fine level averaged onto the coarse level's r (the block
 // sums of k_lin_residual_restrict32), and q with it; the second row's share
 // passes through the fine level's scratch t.  dzero: d = 0.
-__device__ __forceinline__ void tail_restrict(const LvlF& L, const TLev F, const TLev C,
-                                              bool dzero) {
+__device__ __forceinline__ void tail_restrict(const TailParams& P, int l, const TLev F,
+                                              const TLev C, bool dzero) {
+  const LvlF L = P.L[l];
   const int n = L.n, half = n >> 1, nc = half, cs = F.cs, hp = half * n, cells = nc * nc * nc;
-  const TCoarse c(nc);
+  const TCoarse c(nc, P.rhalf[l]);
   float a[4] = {0.f, 0.f, 0.f, 0.f};     // rows, q
   if (c.on) {
     // position I of both colours in row j of the two child planes
@@ -315,22 +327,22 @@ __device__ __forceinline__ void tail_restrict(const LvlF& L, const TLev F, const
 
 // d_F += P d_C (assign: d_F = P d_C): one-dimensional passes z, y, x with
 // weights 3 and 1 as k_prolong_add32.
-__device__ __forceinline__ void tail_prolong(int n, const TLev C, const TLev F, bool assign) {
-  const int half = n >> 1, nc = half, hn = nc >> 1;
-  const TCoarse c(nc);
+__device__ __forceinline__ void tail_prolong(const TailParams& P, int l, const TLev C,
+                                             const TLev F, bool assign) {
+  const int n = P.L[l].n, half = n >> 1, nc = half, hn = nc >> 1;
+  const TCoarse c(nc, P.rhalf[l]);
   if (c.on) {
     const int xs[3] = {c.I == 0 ? nc - 1 : c.I - 1, c.I, c.I + 1 == nc ? 0 : c.I + 1};
     // rows J and the one on the child's side, planes K - 1, K, K + 1
     const int ys[2] = {c.J, c.jj ? (c.J + 1 == nc ? 0 : c.J + 1) : (c.J == 0 ? nc - 1 : c.J - 1)};
     const int zs[3] = {c.K == 0 ? nc - 1 : c.K - 1, c.K, c.K + 1 == nc ? 0 : c.K + 1};
-    int o[3][2][3];
+    // columns x - 1, x, x + 1 of a row whose J + K is even, and odd
+    int ox[2][3];
 #pragma unroll
-    for (int z = 0; z < 3; ++z)
-#pragma unroll
-      for (int y = 0; y < 2; ++y)
-#pragma unroll
-        for (int x = 0; x < 3; ++x)
-          o[z][y][x] = ((xs[x] + ys[y] + zs[z]) & 1) * C.cs + hn * (ys[y] + nc * zs[z]) + (xs[x] >> 1);
+    for (int x = 0; x < 3; ++x) {
+      ox[0][x] = (xs[x] & 1) * C.cs + (xs[x] >> 1);
+      ox[1][x] = (1 - (xs[x] & 1)) * C.cs + (xs[x] >> 1);
+    }
     const int base = c.I + half * (2 * c.J + c.jj + n * 2 * c.K);
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
@@ -341,7 +353,8 @@ __device__ __forceinline__ void tail_prolong(int n, const TLev C, const TLev F, 
 #pragma unroll
         for (int y = 0; y < 2; ++y)
 #pragma unroll
-          for (int x = 0; x < 3; ++x) v[z][y][x] = e[o[z][y][x]];
+          for (int x = 0; x < 3; ++x)
+            v[z][y][x] = e[hn * (ys[y] + nc * zs[z]) + (((ys[y] + zs[z]) & 1) ? ox[1][x] : ox[0][x])];
 #pragma unroll
       for (int kk = 0; kk < 2; ++kk) {
         float y[3];
@@ -381,7 +394,7 @@ __global__ void __launch_bounds__(kTailThreads) k_lin_tail32(TailParams P) {
     float v[2][7][2];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      const int pos = threadIdx.x + s * blockDim.x, row = pos / half;
+      const int pos = threadIdx.x + s * blockDim.x, row = small_div(pos, P.rhalf[0]);
       const size_t g = off + row * n0 + pos - row * half;
       if (pos >= S0.hc) break;
 #pragma unroll
@@ -418,23 +431,23 @@ __global__ void __launch_bounds__(kTailThreads) k_lin_tail32(TailParams P) {
     const int l = s <= last ? s : 2 * last - s;
     const bool down = s < last, coarsest = s == last;
     const TLev S = tlev(P, l);
-    if (s > last) tail_prolong(P.L[l].n, tlev(P, l + 1), S, (dzero >> l) & 1u);
+    if (s > last) tail_prolong(P, l, tlev(P, l + 1), S, (dzero >> l) & 1u);
     const int nu = down ? P.nu1 : P.nu2;
     const int jf = P.kind[l] == PFC_SWEEP_JACOBI ? (l == 0 ? P.jfactor_top : P.jfactor) : 1;
     const int sweeps = coarsest ? P.coarse_sweeps : nu * jf;
     const bool zero = coarsest || (down && (l > 0 || zero_top));
     if (sweeps > 0) {
       if (P.L[l].n % 4 == 0)             // at most 1024 pairs
-        tail_sweeps<true, 1>(P.L[l], P.kind[l], S, sweeps, P.w, zero, coarsest, red, &done);
+        tail_sweeps<true, 1>(P, l, S, sweeps, zero, coarsest, red, &done);
       else                               // n = 14: 1372 positions
-        tail_sweeps<false, 2>(P.L[l], P.kind[l], S, sweeps, P.w, zero, coarsest, red, &done);
+        tail_sweeps<false, 2>(P, l, S, sweeps, zero, coarsest, red, &done);
     } else if (zero) {
       dzero |= 1u << l;
     }
-    if (down) tail_restrict(P.L[l], S, tlev(P, l + 1), (dzero >> l) & 1u);
+    if (down) tail_restrict(P, l, S, tlev(P, l + 1), (dzero >> l) & 1u);
   }
   for (int pos = threadIdx.x; pos < S0.hc; pos += blockDim.x) {
-    const int row = pos / half, g = row * n0 + pos - row * half;
+    const int row = small_div(pos, P.rhalf[0]), g = row * n0 + pos - row * half;
 #pragma unroll
     for (int f = 0; f < 3; ++f)
 #pragma unroll
