@@ -115,15 +115,16 @@ typedef struct pfc_params {
                                 slabs over the CTAs, neighbour planes through
                                 distributed shared memory) where the device
                                 can run such a cluster; 2 uses the cluster
-                                only where the single-block tail would start
-                                (levels of at most 16^3 cells), the levels
-                                above keeping their full-GPU launches (1464
-                                against 1425 steps/s on the 128^3 smooth-mode
-                                workload); 0 (default) keeps separate
-                                launches down to 16^3 and one block below,
-                                faster for ensembles.  Same arithmetic up to
-                                summation order and the approximate division
-                                of the pointwise solve */
+                                only for levels of at most 16^3 cells, and
+                                there only where they do not fit the
+                                single-block tail, which takes less time
+                                (348 against 352 us a step on the 128^3
+                                smooth-mode workload), the levels above
+                                keeping their full-GPU launches; 0 (default)
+                                keeps separate launches down to 16^3 and one
+                                block below, faster for ensembles.  Same
+                                arithmetic up to summation order and the
+                                approximate division of the pointwise solve */
   int    step_diagnostics;   /* 1: every step also forms the energy/mass sums
                                 of its new state in the same graph launch
                                 (no further launch or synchronisation), and
