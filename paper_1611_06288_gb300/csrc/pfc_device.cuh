@@ -314,4 +314,30 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* smem /* 32*NV
   __syncthreads();
 }
 
+// The same for several components, through NV * blockDim.x doubles of shared
+// memory (blocks of whole warps, at most 32): warp c % warps sums component c,
+// first lane by lane over the warps' rows, then in a shuffle tree.  A warp's
+// FP64 add holds the FP64 pipe for 16 clocks whatever its lanes add; this takes
+// NV (warps + 4) of them, block_sum 5 NV (warps + 1).
+template <int NV>
+__device__ __forceinline__ void block_sum_rows(double (&v)[NV], double* smem) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nt = blockDim.x, nw = nt >> 5;
+#pragma unroll
+  for (int c = 0; c < NV; ++c) smem[c * nt + threadIdx.x] = v[c];
+  __syncthreads();
+  for (int c = wid; c < NV; c += nw) {
+    double x = smem[c * nt + lane];
+    for (int w = 1; w < nw; ++w) x += smem[c * nt + w * 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) smem[c * nt] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int c = 0; c < NV; ++c) v[c] = smem[c * nt];
+  }
+}
+
 }  // namespace pfc

@@ -695,7 +695,7 @@ __global__ void k_reduce_final(const double* __restrict__ partials, int nparts,
                                double* out) {
   pdl_wait();
   pdl_trigger();
-  __shared__ double sm[32 * NV];
+  __shared__ double sm[kReduceThreads * NV];
   partials += (size_t)blockIdx.x * nparts * NV;
   out += (size_t)blockIdx.x * kReduceComps;
   double acc[NV];
@@ -705,7 +705,7 @@ __global__ void k_reduce_final(const double* __restrict__ partials, int nparts,
 #pragma unroll
     for (int c = 0; c < NV; ++c) acc[c] += partials[(int64_t)p * NV + c];
   }
-  block_sum<NV>(acc, sm);
+  block_sum_rows<NV>(acc, sm);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int c = 0; c < NV; ++c) out[c] = acc[c];
@@ -717,7 +717,7 @@ __global__ void k_reduce_final(const double* __restrict__ partials, int nparts,
 // reusing the Laplacian that ||Delta_h a||^2 needs.
 __global__ void k_diagnostics(int n, const double* __restrict__ a,
                               const double* __restrict__ b, double* partials) {
-  __shared__ double sm[32 * 6];
+  __shared__ double sm[kReduceThreads * 6];
   const int cells = n * n * n;
   double acc[6] = {0, 0, 0, 0, 0, 0};
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cells; t += gridDim.x * blockDim.x) {
@@ -737,11 +737,19 @@ __global__ void k_diagnostics(int n, const double* __restrict__ a,
     acc[4] = fma(ex, ex, fma(ey, ey, fma(ez, ez, acc[4])));
     acc[5] += x;
   }
-  block_sum<6>(acc, sm);
+  block_sum_rows<6>(acc, sm);
   if (threadIdx.x == 0) {
     for (int c = 0; c < 6; ++c) partials[(int64_t)blockIdx.x * 6 + c] = acc[c];
   }
 }
+
+// Blocks of k_diagnostics_cached an SM holds, and gets, over all members.
+// With 16 loads a thread in flight and the sums by rows: two 31.6 us at 128^3
+// and 195 at 256^3, three 29.4 and 174, four 30.6 and 182 (its 64 registers
+// spill); with shuffle trees and two, 35.6 and 201.  The 5 FP64 operations and
+// 2 conversions a cell hold the FP64 pipe for 20 and 160 us.
+constexpr int kDiagPerSM = 3;
+constexpr int kDiagBlocks = kDiagPerSM * 152;
 
 // The raw sums of k_diagnostics from the stored unscaled Laplacians of a and
 // b: -(a, Lap a) and (Lap a)^2 directly, and the forward-face sum of
@@ -753,13 +761,13 @@ __global__ void k_diagnostics(int n, const double* __restrict__ a,
 // below 2^54 each: no overflow); larger values take the FP64 adds.  The two
 // differences a - b and Lap a - Lap b are formed from the same images (exact,
 // one rounding each), which leaves 5 FP64 operations per cell.
-__global__ void k_diagnostics_cached(int n, const double* __restrict__ a,
-                                     const double* __restrict__ b,
-                                     const double* __restrict__ lapa,
-                                     const double* __restrict__ lapb, double* partials) {
+__global__ void __launch_bounds__(kReduceThreads, kDiagPerSM)
+    k_diagnostics_cached(int n, const double* __restrict__ a, const double* __restrict__ b,
+                         const double* __restrict__ lapa, const double* __restrict__ lapb,
+                         double* partials) {
   pdl_wait();
   pdl_trigger();
-  __shared__ double sm[32 * 6];
+  __shared__ double sm[kReduceThreads * 6];
   const int cells = n * n * n;
   const size_t off = (size_t)blockIdx.y * cells;     // member of an ensemble
   a += off, b += off, lapa += off, lapb += off;
@@ -811,7 +819,7 @@ __global__ void k_diagnostics_cached(int n, const double* __restrict__ a,
   for (; t < cells; t += stride) cell(__ldg(a + t), __ldg(lapa + t), __ldg(b + t), __ldg(lapb + t));
   acc[5] += fix_to_double(s1);
   acc[1] += fix_to_double(s2);
-  block_sum<6>(acc, sm);
+  block_sum_rows<6>(acc, sm);
   if (threadIdx.x == 0) {
     for (int c = 0; c < 6; ++c) partials[(int64_t)blockIdx.x * 6 + c] = acc[c];
   }
@@ -907,7 +915,7 @@ __global__ void k_reduce_final_state(const double* __restrict__ partials, int np
   pdl_wait();
   pdl_trigger();
   constexpr int NV = 6;
-  __shared__ double sm[32 * NV];
+  __shared__ double sm[kReduceThreads * NV];
   partials += (size_t)blockIdx.x * nparts * NV;
   out += (size_t)blockIdx.x * kReduceComps;
   double acc[NV];
@@ -917,19 +925,13 @@ __global__ void k_reduce_final_state(const double* __restrict__ partials, int np
 #pragma unroll
     for (int c = 0; c < NV; ++c) acc[c] += partials[(int64_t)p * NV + c];
   }
-  block_sum<NV>(acc, sm);
+  block_sum_rows<NV>(acc, sm);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int c = 0; c < NV; ++c) out[c] = acc[c];
     state_out[blockIdx.x] = state[blockIdx.x];
   }
 }
-
-// Blocks of k_diagnostics_cached over all members: two per SM.  Its six
-// FP64 block sums cost 5 lanes of FP64 adds per thread in the warp
-// shuffles, as much as its per-cell work when a thread has only 7 cells
-// (1216 blocks at 128^3), so each thread takes about 27.
-constexpr int kDiagBlocks = 2 * 152;
 
 cudaError_t launch_diagnostics_cached(int n, const double* a, const double* b,
                                       const double* lapa, const double* lapb, double* partials,
