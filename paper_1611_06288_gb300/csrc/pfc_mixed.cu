@@ -1278,10 +1278,11 @@ __device__ __forceinline__ float2 nbsum2(float2 o, float e, bool sg, float2 y0, 
 // half-row) of its cells, the rows beside them and the x neighbours beyond.
 struct MarchCell {
   size_t moff;
-  int k0, k1, j, c, ym, yp, xl, xr;
+  int k0, k1, j, p, c, ym, yp, xl, xr;
   bool on;
   __device__ __forceinline__ MarchCell(int n, int zc) {
-    const int half = n >> 1, p = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int half = n >> 1;
+    p = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     int zb = blockIdx.z;
     moff = (size_t)member_of(zb, (n + zc - 1) / zc) * n * n * n;
     j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1421,19 +1422,39 @@ __global__ void k_lin_jacobi32(LvlF L, float w, const float* __restrict__ d1,
 }
 
 
-// The marching sweep: both colours of two positions per thread.
+// u += d on the four natural cells 2p .. 2p + 3 of a row, as k_correct64 adds
+// them (u 16-byte aligned).
+__device__ __forceinline__ void add4(double* u, float v0, float v1, float v2, float v3) {
+  double2* const up = reinterpret_cast<double2*>(u);
+  double2 lo = up[0], hi = up[1];
+  lo.x += f2d(v0);
+  lo.y += f2d(v1);
+  hi.x += f2d(v2);
+  hi.y += f2d(v3);
+  up[0] = lo;
+  up[1] = hi;
+}
+
+// The marching sweep: both colours of two positions per thread.  U = float:
+// the new values go to t.  U = double, the last sweep of a correction's last
+// V-cycle on a Jacobi finest level: they are added to the state u (t1 .. t3)
+// instead, which saves their way through memory (24 B a cell) and a launch.
+// Against the sweep and k_correct64, us: 96^3 14.2 / 18.1, 256^3 219 / 298,
+// 42 x 64^3 146 / 196.
+template <class U>
 __global__ void __launch_bounds__(128, 4) k_lin_jacobi32m(
     LvlF L, float w, int zc, const float* __restrict__ d1, const float* __restrict__ d2,
-    const float* __restrict__ d3, float* __restrict__ t1, float* __restrict__ t2,
-    float* __restrict__ t3, const float* __restrict__ r1, const float* __restrict__ r2,
-    const float* __restrict__ r3, const float* __restrict__ q) {
+    const float* __restrict__ d3, U* __restrict__ t1, U* __restrict__ t2, U* __restrict__ t3,
+    const float* __restrict__ r1, const float* __restrict__ r2, const float* __restrict__ r3,
+    const float* __restrict__ q) {
+  constexpr bool kAdd = !std::is_same<U, float>::value;
   pdl_wait();
   pdl_trigger();
   const int n = L.n, half = n >> 1, nn = n * n;
   const MarchCell M(n, zc);
   if (!M.on) return;
   const float* const d[3] = {d1 + M.moff, d2 + M.moff, d3 + M.moff};
-  float* const t[3] = {t1 + M.moff, t2 + M.moff, t3 + M.moff};
+  U* const t[3] = {t1 + M.moff, t2 + M.moff, t3 + M.moff};
   const float* const rq[4] = {r1 + M.moff, r2 + M.moff, r3 + M.moff, q + M.moff};
   const float2 ww = f2_all(w);
   float2 zm[3][2], zc_[3][2];
@@ -1466,15 +1487,24 @@ __global__ void __launch_bounds__(128, 4) k_lin_jacobi32m(
                            ldg2(o + M.yp), zm[f][1 - c], zp[f][1 - c]);
       }
     }
+    float2 x[3][2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      float2 x[3];
-      lin_point2(L, sum[0][c], sum[1][c], sum[2][c], v[3][c], v[0][c], v[1][c], v[2][c], x[0],
-                 x[1], x[2]);
+      lin_point2(L, sum[0][c], sum[1][c], sum[2][c], v[3][c], v[0][c], v[1][c], v[2][c], x[0][c],
+                 x[1][c], x[2][c]);
 #pragma unroll
-      for (int f = 0; f < 3; ++f)
-        *reinterpret_cast<float2*>(t[f] + g + c * half + M.c) =
-            f2_fma(ww, f2_sub(x[f], zc_[f][c]), zc_[f][c]);
+      for (int f = 0; f < 3; ++f) {
+        x[f][c] = f2_fma(ww, f2_sub(x[f][c], zc_[f][c]), zc_[f][c]);
+        if constexpr (!kAdd) *reinterpret_cast<float2*>(t[f] + g + c * half + M.c) = x[f][c];
+      }
+    }
+    if constexpr (kAdd) {
+      // natural cells 2p .. 2p + 3: colour 0 first where its offset is 0
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const float2 a = sg ? x[f][1] : x[f][0], b = sg ? x[f][0] : x[f][1];
+        add4(t[f] + g + M.c + M.p, a.x, b.x, a.y, b.y);
+      }
     }
 #pragma unroll
     for (int f = 0; f < 3; ++f)
@@ -1516,17 +1546,17 @@ __global__ void k_lin_jacobi32_zero(LvlF L, float w, float* __restrict__ t1,
 // cells at the same positions of the other half are the four consecutive
 // natural cells 2 p0 .. 2 p0 + 3 of the row (which of each pair comes first
 // depends on the row's colour offset), so u moves as two 16-byte vectors per
-// component.  Same sums and solve as the pass, same u + f2d(d) as
-// k_correct64: u equals the two launches bit for bit.  d's colour-1 cells
-// are left as they were.
+// component.  Same sums and solve as the pass, same u + d as k_correct64: u
+// equals the two launches bit for bit.  d's colour-1 cells are left as they
+// were.
 __global__ void k_lin_smooth32_correct(LvlF L, const float* __restrict__ d1,
-                                         const float* __restrict__ d2,
-                                         const float* __restrict__ d3,
-                                         const float* __restrict__ r1,
-                                         const float* __restrict__ r2,
-                                         const float* __restrict__ r3,
-                                         const float* __restrict__ q, double* __restrict__ u1,
-                                         double* __restrict__ u2, double* __restrict__ u3) {
+                                       const float* __restrict__ d2,
+                                       const float* __restrict__ d3,
+                                       const float* __restrict__ r1,
+                                       const float* __restrict__ r2,
+                                       const float* __restrict__ r3,
+                                       const float* __restrict__ q, double* __restrict__ u1,
+                                       double* __restrict__ u2, double* __restrict__ u3) {
   pdl_wait();
   pdl_trigger();
   const int n = L.n, half = n >> 1;
@@ -1577,16 +1607,8 @@ __global__ void k_lin_smooth32_correct(LvlF L, const float* __restrict__ d1,
 #pragma unroll
   for (int q3 = 0; q3 < 3; ++q3) {
     // natural order 2 p0 .. 2 p0 + 3: colour 1 first when sigma = 0
-    const float v0 = sigma ? a[q3].x : nd[q3].x, v1 = sigma ? nd[q3].x : a[q3].x;
-    const float v2 = sigma ? a[q3].y : nd[q3].y, v3 = sigma ? nd[q3].y : a[q3].y;
-    double2* const up = reinterpret_cast<double2*>(u[q3] + row + 2 * p0);
-    double2 lo = up[0], hi = up[1];
-    lo.x += f2d(v0);
-    lo.y += f2d(v1);
-    hi.x += f2d(v2);
-    hi.y += f2d(v3);
-    up[0] = lo;
-    up[1] = hi;
+    const float2 x = sigma ? a[q3] : nd[q3], y = sigma ? nd[q3] : a[q3];
+    add4(u[q3] + row + 2 * p0, x.x, y.x, x.y, y.y);
   }
 }
 
@@ -3352,10 +3374,11 @@ struct Ctx32 {
 };
 
 // `sweeps` damped Jacobi sweeps d -> t -> d ...; *in_t: whether the iterate is
-// in t, on entry and on return.
+// in t, on entry and on return.  u (n % 4 == 0, not for the sweep from zero):
+// the last sweep adds to u instead.
 cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* const* d,
                      float* const* t, float* const* r, const float* q, cudaStream_t st,
-                     bool pdl, int nb, bool* in_t) {
+                     bool pdl, int nb, bool* in_t, double* const* u = nullptr) {
   const int n = L.n;
   const bool pairs = n % 4 == 0;                // two cells per thread, float2 moves
   const Launch3 g = launch3(pairs ? n / 2 : n, n, n * nb);
@@ -3374,8 +3397,11 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
     if (pairs && z)
       e = launch_k(pdl, k_lin_jacobi32_zero, g.grid, g.block, 0, st, L, w, dst[0], dst[1], dst[2],
                    r[0], r[1], r[2], q);
+    else if (u && done + 1 == sweeps)
+      e = launch_k(pdl, k_lin_jacobi32m<double>, mg.grid, mg.block, 0, st, L, w, mg.zc, src[0],
+                   src[1], src[2], u[0], u[1], u[2], r[0], r[1], r[2], q);
     else if (pairs)
-      e = launch_k(pdl, k_lin_jacobi32m, mg.grid, mg.block, 0, st, L, w, mg.zc, src[0], src[1],
+      e = launch_k(pdl, k_lin_jacobi32m<float>, mg.grid, mg.block, 0, st, L, w, mg.zc, src[0], src[1],
                    src[2], dst[0], dst[1], dst[2], r[0], r[1], r[2], q);
     else
       e = launch_k(pdl, z ? k_lin_jacobi32<true> : k_lin_jacobi32<false>, g.grid, g.block, 0,
@@ -3392,10 +3418,21 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
 }
 
 // jacobi32 on level l of a cycle: where the result is in t, d and t change
-// places (the cycle's own pointers), so no copy follows an odd count.
-cudaError_t jacobi_level32(const Ctx32& c, int l, int sweeps, bool zero_init, bool in_t) {
-  cudaError_t e = jacobi32(c.L[l], sweeps, c.w, zero_init, c.mx->d[l], c.mx->t[l], c.mx->r[l],
-                           c.mx->q[l], c.st, c.pr == nullptr, c.nb, &in_t);
+// places (the cycle's own pointers), so no copy follows an odd count.  fold:
+// the last sweep adds to c.fold_u (n % 4 == 0).
+cudaError_t jacobi_level32(const Ctx32& c, int l, int sweeps, bool zero_init, bool in_t,
+                           bool fold = false) {
+  prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
+  cudaError_t e = jacobi32(c.L[l], fold ? sweeps - 1 : sweeps, c.w, zero_init, c.mx->d[l],
+                           c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st, c.pr == nullptr, c.nb, &in_t);
+  prof_end(c.pr, PFC_K_LIN_SMOOTH, l, fold ? sweeps - 1 : sweeps, c.st);
+  if (fold && e == cudaSuccess) {
+    // timed as the correction it replaces
+    prof_begin(c.pr, PFC_K_CORRECT, c.st);
+    e = jacobi32(c.L[l], 1, c.w, false, c.mx->d[l], c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st,
+                 c.pr == nullptr, c.nb, &in_t, c.fold_u);
+    prof_end(c.pr, PFC_K_CORRECT, l, 1, c.st);
+  }
   if (in_t)
     for (int f = 0; f < 3; ++f) {
       float* const x = c.mx->d[l][f];
@@ -3438,25 +3475,22 @@ cudaError_t rb_pass32_correct(const Ctx32& c, int l) {
 }
 
 // Whether a correction's u += d can fold into the finest level's last
-// post-smoothing pass: a red-black finest level with post-smoothing, wide
-// enough that no tail launch takes it (more than 32 cells), its rows a
-// multiple of four cells (the paired pass).
+// post-smoothing pass: a finest level with post-smoothing, wide enough that no
+// tail launch takes it (more than 32 cells), its rows a multiple of four cells
+// (the paired passes).
 bool correction_folds(const Ctx32& c) {
-  return c.nl >= 2 && c.kind[0] == PFC_SWEEP_RB && c.p->nu2 > 0 && c.L[0].n > kCtMaxN &&
-         c.L[0].n % 4 == 0;
+  return c.nl >= 2 && c.p->nu2 > 0 && (c.kind[0] != PFC_SWEEP_JACOBI || c.jfactor0 > 0) &&
+         c.L[0].n > kCtMaxN && c.L[0].n % 4 == 0;
 }
 
-// `sweeps` post- (or pre-) smoothing sweeps on level l; fold: the last
-// colour-1 pass adds the result to c.fold_u (red-black, n % 4 == 0).
+// `sweeps` post- (or pre-) smoothing sweeps on level l; fold: the last pass
+// adds the result to c.fold_u (n % 4 == 0).
 cudaError_t smooth32(const Ctx32& c, int l, int sweeps, bool zero_init, bool fold = false) {
   if (sweeps <= 0) return cudaSuccess;
+  if (c.kind[l] == PFC_SWEEP_JACOBI)
+    return jacobi_level32(c, l, sweeps * (l == 0 ? c.jfactor0 : c.jfactor), zero_init, false,
+                          fold);
   prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
-  if (c.kind[l] == PFC_SWEEP_JACOBI) {
-    const int js = sweeps * (l == 0 ? c.jfactor0 : c.jfactor);
-    cudaError_t e = jacobi_level32(c, l, js, zero_init, false);
-    prof_end(c.pr, PFC_K_LIN_SMOOTH, l, js, c.st);
-    return e;
-  }
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < sweeps && e == cudaSuccess; ++s)
     for (int colour = 0; colour < 2 && e == cudaSuccess; ++colour)
@@ -3515,10 +3549,7 @@ cudaError_t prolong_smooth32(const Ctx32& c, int l, bool assign, int sweeps) {
   if (e != cudaSuccess) return e;
   if (jacobi) {
     // the first sweep left its result in t
-    prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
-    e = jacobi_level32(c, l, sweeps - 1, false, true);
-    prof_end(c.pr, PFC_K_LIN_SMOOTH, l, sweeps - 1, c.st);
-    return e;
+    return jacobi_level32(c, l, sweeps - 1, false, true, l == 0 && c.fold_u != nullptr);
   }
   prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
   e = rb_pass32(c, l, 1, false);
@@ -3785,8 +3816,9 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
   // pass formed every colour-1 value of its tile and halo per cell (25 us
   // per launch at 128^3 against 6.1 + 6.5 us for the prolongation's
   // coarse-column carry and the plain pass)
+  const bool fold = l == 0 && c.fold_u != nullptr;
   if (c.kind[l] == PFC_SWEEP_JACOBI && prolong_fuses(L.n, post) &&
-      prolong_fuse_pays(L.n, c.nb, dzero))
+      prolong_fuse_pays(L.n, c.nb, dzero) && !(fold && post == 1))
     return prolong_smooth32(c, l, dzero, post);
   const int pz = prolong_planes(nc, 3 * c.nb);
   // a red-black post-smoothing pass of colour 0 comes next: it recomputes
@@ -3798,7 +3830,7 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
                mx.d[l + 1][2], mx.d[l][0], mx.d[l][1], mx.d[l][2]);
   prof_end(c.pr, PFC_K_LIN_PROLONG, l, 1, c.st);
   if (e != cudaSuccess) return e;
-  return smooth32(c, l, c.p->nu2, false, l == 0 && c.fold_u != nullptr);
+  return smooth32(c, l, c.p->nu2, false, fold);
 }
 
 }  // namespace
@@ -4372,6 +4404,8 @@ cudaError_t mixed_vcycles(MixedBufs& mx, const pfc_params& p, int nl, const int*
     l += 1 + extra;
   }
   *folded = u != nullptr && p.inner_cycles > 0 && correction_folds(c);
+  // 16-byte moves of u: the adjoint's is the caller's and may start at any element
+  for (int f = 0; f < 3 && *folded; ++f) *folded = (uintptr_t)u[f] % 16 == 0;
   for (int ic = 0; ic < p.inner_cycles && e == cudaSuccess; ++ic) {
     c.fold_u = (*folded && ic + 1 == p.inner_cycles) ? u : nullptr;
     e = vcycle32(c, 0, ic == 0);
