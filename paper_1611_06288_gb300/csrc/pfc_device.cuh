@@ -265,11 +265,14 @@ __device__ __forceinline__ void point_solve(const Lvl& L, double sphi, double sm
 }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream
-// serialization may be scheduled while its predecessor drains; pdl_wait()
-// blocks until the predecessor has completed and its writes are visible (a
-// no-op for a normal launch), pdl_trigger() lets the successor be scheduled.
+// serialization may be set up while its predecessor drains; pdl_wait() blocks
+// until the predecessor has completed and its writes are visible (a no-op for a
+// normal launch).  No kernel lets its successor in early: blocks that wait for
+// it hold slots of the SMs it still runs on.  ms of a run, without programmatic
+// launches / with an early launch_dependents in each kernel / as it is: 128^3
+// FP64 17.0 / 18.8 / 17.2, 32^3 FP64 7.7 / 7.4 / 7.4, 64^3 gradient 78 / 67 /
+// 66, 96^3 growth 12.4 / 12.6 / 12.2.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
 // Launch with programmatic stream serialization when `pdl` is set (the
 // kernel must call pdl_wait() before it reads what its predecessor wrote).

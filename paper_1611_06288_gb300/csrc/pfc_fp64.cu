@@ -83,7 +83,6 @@ __global__ void k_guess_all(int64_t cells, int extrap, const double* __restrict_
                             const double* __restrict__ o0, double* m1, double* o1,
                             double* __restrict__ phi) {
   pdl_wait();
-  pdl_trigger();
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cells;
        t += (int64_t)gridDim.x * blockDim.x) {
     const double bb = __ldg(b + t), mm = __ldg(m0 + t), oo = __ldg(o0 + t);
@@ -141,7 +140,6 @@ __global__ void k_source_cached(Lvl L, int members, const double* __restrict__ c
                                 const double* __restrict__ lapb, const double* __restrict__ lapc,
                                 double* __restrict__ S2, double* __restrict__ S3) {
   pdl_wait();
-  pdl_trigger();
   const int64_t cells = (int64_t)L.n * L.n * L.n;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= cells * members) return;
@@ -164,7 +162,6 @@ __global__ void k_smooth_colour(Lvl L, int colour, double* phi, double* mu, doub
                                 const double* __restrict__ S3,
                                 const double* __restrict__ b) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, half = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)half * n * n) return;
@@ -195,7 +192,6 @@ __global__ void k_jacobi64(Lvl L, double w, const double* __restrict__ phi,
                            const double* __restrict__ S2, const double* __restrict__ S3,
                            const double* __restrict__ b) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n * n) return;
@@ -255,7 +251,6 @@ __global__ void k_residual_restrict8(Lvl L, const double* __restrict__ phi,
                                      double* __restrict__ uc3, double* __restrict__ wc1,
                                      double* __restrict__ wc2, double* __restrict__ wc3) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, nc = n >> 1;
   const int64_t cells = (int64_t)nc * nc * nc;
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -345,7 +340,6 @@ __global__ void __launch_bounds__(128) k_residual_restrict(
     double* __restrict__ uc2, double* __restrict__ uc3, double* __restrict__ wc1,
     double* __restrict__ wc2, double* __restrict__ wc3) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, nc = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nc * nc * nc) return;
@@ -384,7 +378,6 @@ __global__ void __launch_bounds__(128) k_residual_restrict(
 
 __global__ void k_restrict(int n, const double* __restrict__ f, double* __restrict__ c) {
   pdl_wait();
-  pdl_trigger();
   const int nc = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nc * nc * nc) return;
@@ -408,7 +401,6 @@ __global__ void k_coarse_source(Lvl L, const double* __restrict__ u1,
                                 const double* __restrict__ bc, double* r1, double* r2,
                                 double* r3) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n * n) return;
@@ -448,7 +440,6 @@ __global__ void k_prolong_add(int n, const double* __restrict__ v1, const double
                               double* __restrict__ u1, double* __restrict__ u2,
                               double* __restrict__ u3) {
   pdl_wait();
-  pdl_trigger();
   const int nc = n >> 1, f = blockIdx.y;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n * n) return;
@@ -490,7 +481,6 @@ __global__ void __launch_bounds__(kPfI * kPfJ) k_prolong_add_tile(
     const double* __restrict__ w3, double* __restrict__ u1, double* __restrict__ u2,
     double* __restrict__ u3) {
   pdl_wait();
-  pdl_trigger();
   constexpr int W = kPfI + 2, H = kPfJ + 2;
   __shared__ double sh[2][2][H][W];          // [buffer][child in z][y][x]
   const int nc = n >> 1, chunks = (nc + zc - 1) / zc;
@@ -589,7 +579,6 @@ __global__ void k_coarse_solve(Lvl L, int kind, double w, int max_sweeps, int sh
                                double* t3, const double* S1, const double* S2, const double* S3,
                                const double* b) {
   pdl_wait();
-  pdl_trigger();
   extern __shared__ double cs[];
   const int n = L.n, half = n >> 1;
   const int ncell = n * n * n;
@@ -669,7 +658,6 @@ __global__ void k_residual_norm2(Lvl L, const double* __restrict__ phi,
                                  const double* __restrict__ b, double* partials,
                                  double* __restrict__ lap) {
   pdl_wait();
-  pdl_trigger();
   __shared__ double sm[32];
   const int n = L.n;
   const int64_t cells = (int64_t)n * n * n;
@@ -694,7 +682,6 @@ template <int NV>
 __global__ void k_reduce_final(const double* __restrict__ partials, int nparts,
                                double* out) {
   pdl_wait();
-  pdl_trigger();
   __shared__ double sm[kReduceThreads * NV];
   partials += (size_t)blockIdx.x * nparts * NV;
   out += (size_t)blockIdx.x * kReduceComps;
@@ -766,7 +753,6 @@ __global__ void __launch_bounds__(kReduceThreads, kDiagPerSM)
                          const double* __restrict__ lapa, const double* __restrict__ lapb,
                          double* partials) {
   pdl_wait();
-  pdl_trigger();
   __shared__ double sm[kReduceThreads * 6];
   const int cells = n * n * n;
   const size_t off = (size_t)blockIdx.y * cells;     // member of an ensemble
@@ -831,7 +817,6 @@ __global__ void k_decide(cudaGraphConditionalHandle handle, int use_handle,
                          const double* sum, StepState* s, int members, double inv_3n3,
                          double tol, int max_iter, int first) {
   pdl_wait();
-  pdl_trigger();
   // one thread per ensemble member (sum[m] its sum of squared residuals);
   // a member that has converged stays converged, and the loop runs while
   // some member is still running and none has failed
@@ -913,7 +898,6 @@ __global__ void k_reduce_final_state(const double* __restrict__ partials, int np
                                      double* out, const StepState* __restrict__ state,
                                      StepState* state_out) {
   pdl_wait();
-  pdl_trigger();
   constexpr int NV = 6;
   __shared__ double sm[kReduceThreads * NV];
   partials += (size_t)blockIdx.x * nparts * NV;

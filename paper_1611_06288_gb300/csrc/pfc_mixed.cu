@@ -330,7 +330,6 @@ __global__ void __launch_bounds__(kFxTX * kFxTY, 4) k_defect64_fx(
     double* __restrict__ lap, const double* __restrict__ c1m, double* __restrict__ lapmu,
     double* __restrict__ lapom) {
   pdl_wait();
-  pdl_trigger();
   extern __shared__ int64_t ring[];   // [kFxRing][3][kFxTY + 2][kFxTX + 2]
   __shared__ float sm[32];
   constexpr int TW = kFxTX + 2, TP = (kFxTY + 2) * TW, TS = 3 * TP;
@@ -472,7 +471,6 @@ __global__ void __launch_bounds__(256) k_defect64_point(
     float* __restrict__ r2, float* __restrict__ r3, float* __restrict__ q, double* partials,
     double* __restrict__ lap, const double* __restrict__ c1m) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -522,7 +520,6 @@ __global__ void __launch_bounds__(256) k_start64_point(
     float* __restrict__ r3, float* __restrict__ q, double* partials, double* __restrict__ lap,
     const double* __restrict__ c1m) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -600,7 +597,6 @@ __global__ void __launch_bounds__(256, 4) k_start64_extrap(
     float* __restrict__ r3, float* __restrict__ q, double* partials,
     double* __restrict__ lap, const double* __restrict__ c1m) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -1108,7 +1104,6 @@ __global__ void k_df_to_f64(int64_t count, const float2* y, double* x) {
 // Fixed-order sum of each member's partials (one block per member): out[m].
 __global__ void k_reduce1(const double* __restrict__ partials, int nparts, double* out) {
   pdl_wait();
-  pdl_trigger();
   __shared__ double sm[32];
   const int m = blockIdx.x;
   partials += (size_t)m * nparts;
@@ -1124,7 +1119,6 @@ __global__ void k_reduce1(const double* __restrict__ partials, int nparts, doubl
 __global__ void k_reduce1_decide(const double* __restrict__ partials, int nparts, double* out,
                                  DecideArgs a) {
   pdl_wait();
-  pdl_trigger();
   __shared__ double sm[32];
   double acc[1] = {0.0};
   for (int p = threadIdx.x; p < nparts; p += blockDim.x) acc[0] += partials[p];
@@ -1140,7 +1134,6 @@ __global__ void k_reduce1_decide(const double* __restrict__ partials, int nparts
 // 8-cell average of a split-layout field onto the (split-layout) level n/2.
 __global__ void k_restrict32(int n, const float* __restrict__ f, float* __restrict__ c) {
   pdl_wait();
-  pdl_trigger();
   const int nc = n >> 1;
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   int K = blockIdx.z;
@@ -1226,7 +1219,6 @@ __global__ void k_lin_smooth32(LvlF L, int colour, float* d1, float* d2, float* 
                                const float* __restrict__ r1, const float* __restrict__ r2,
                                const float* __restrict__ r3, const float* __restrict__ q) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, half = n >> 1;
   const int p = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z;
@@ -1324,7 +1316,6 @@ __global__ void __launch_bounds__(128, 6) k_lin_smooth32m(
     LvlF L, int colour, int zc, float* d1, float* d2, float* d3, const float* __restrict__ r1,
     const float* __restrict__ r2, const float* __restrict__ r3, const float* __restrict__ q) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, half = n >> 1, nn = n * n;
   const MarchCell M(n, zc);
   if (!M.on) return;
@@ -1368,7 +1359,6 @@ __global__ void k_lin_smooth32_zero(LvlF L, float* __restrict__ d1, float* __res
                                     const float* __restrict__ r2, const float* __restrict__ r3,
                                     const float* __restrict__ q) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n;
   const int p = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1394,7 +1384,6 @@ __global__ void k_lin_jacobi32(LvlF L, float w, const float* __restrict__ d1,
                                const float* __restrict__ r2, const float* __restrict__ r3,
                                const float* __restrict__ q) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, half = n >> 1;
   const int x = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z;
@@ -1449,7 +1438,6 @@ __global__ void __launch_bounds__(128, 4) k_lin_jacobi32m(
     const float* __restrict__ q) {
   constexpr bool kAdd = !std::is_same<U, float>::value;
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, half = n >> 1, nn = n * n;
   const MarchCell M(n, zc);
   if (!M.on) return;
@@ -1522,7 +1510,6 @@ __global__ void k_lin_jacobi32_zero(LvlF L, float w, float* __restrict__ t1,
                                     const float* __restrict__ r1, const float* __restrict__ r2,
                                     const float* __restrict__ r3, const float* __restrict__ q) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n;
   const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1558,7 +1545,6 @@ __global__ void k_lin_smooth32_correct(LvlF L, const float* __restrict__ d1,
                                        const float* __restrict__ q, double* __restrict__ u1,
                                        double* __restrict__ u2, double* __restrict__ u3) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, half = n >> 1;
   const int p0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1616,7 +1602,6 @@ __global__ void k_copy3(int cells, const float* __restrict__ a1, const float* __
                         const float* __restrict__ a3, float* __restrict__ b1,
                         float* __restrict__ b2, float* __restrict__ b3) {
   pdl_wait();
-  pdl_trigger();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= cells) return;
   b1[t] = a1[t];
@@ -1696,7 +1681,6 @@ __global__ void k_lin_residual_restrict32(LvlF L, const float* __restrict__ d1,
                                           float* __restrict__ c1, float* __restrict__ c2,
                                           float* __restrict__ c3) {
   pdl_wait();
-  pdl_trigger();
   const int n = L.n, nc = n >> 1;
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   int K = blockIdx.z;
@@ -1765,7 +1749,6 @@ __global__ void __launch_bounds__(kChTX * kChTY * kChTZ) k_lin_restrict_chain32(
     float* __restrict__ e2, float* __restrict__ e3, float* __restrict__ g1,
     float* __restrict__ g2, float* __restrict__ g3) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float s1[3][kChTZ][kChTY][kChTX];
   __shared__ float s2[3][kChTZ / 2][kChTY / 2][kChTX / 2];
   const int n = L.n, nc = n >> 1;
@@ -1884,7 +1867,6 @@ __global__ void __launch_bounds__(kChTX * kChTY * kChTZ) k_restrict_chain32(
     int n, const float* __restrict__ f, float* __restrict__ c, float* __restrict__ e,
     float* __restrict__ g) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float s1[kChTZ][kChTY][kChTX];
   __shared__ float s2[kChTZ / 2][kChTY / 2][kChTX / 2];
   const int nc = n >> 1;
@@ -1958,7 +1940,6 @@ __global__ void __launch_bounds__(kPrTI * kPrTJ) k_prolong_add32(
     const float* __restrict__ e3, float* __restrict__ d1, float* __restrict__ d2,
     float* __restrict__ d3) {
   pdl_wait();
-  pdl_trigger();
   constexpr int kW = kPrTI + 2;
   __shared__ float sh[kPrZ + 2][kPrTJ + 2][kW];
   const int nc = n >> 1, half = n >> 1, hc = nc >> 1;
@@ -2174,7 +2155,6 @@ __global__ void __launch_bounds__(kPsTX * TY) k_lin_prolong_sweep32(
     float* __restrict__ t2, float* __restrict__ t3, const float* __restrict__ r1,
     const float* __restrict__ r2, const float* __restrict__ r3, const float* __restrict__ q) {
   pdl_wait();
-  pdl_trigger();
   using T = PsTile<TY, TZ>;
   constexpr int TX = T::TX, NT = T::NT, FX = T::FX, FY = T::FY, FZ = T::FZ;
   constexpr int CX = T::CX, CY = T::CY;
@@ -3210,7 +3190,6 @@ __device__ void ct_prolong(const cg::cluster_group& cl, unsigned me, float* smem
 
 __global__ void __launch_bounds__(kCtThreads, 1) k_lin_ctail32(CTailParams P) {
   pdl_wait();
-  pdl_trigger();
   extern __shared__ float smem[];
   __shared__ float red[2][32];
   __shared__ float cmax[2];
@@ -3310,7 +3289,6 @@ __global__ void k_correct64(int n, double* __restrict__ u1, double* __restrict__
                             double* __restrict__ u3, const float* __restrict__ d1,
                             const float* __restrict__ d2, const float* __restrict__ d3) {
   pdl_wait();
-  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z;
   const size_t off = (size_t)member_of(k, n) * n * n * n;
@@ -3328,7 +3306,6 @@ __global__ void k_correct_df(int n, float2* __restrict__ u1, float2* __restrict_
                              float2* __restrict__ u3, const float* __restrict__ d1,
                              const float* __restrict__ d2, const float* __restrict__ d3) {
   pdl_wait();
-  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
             k = blockIdx.z;
   if (i >= n || j >= n) return;
@@ -3369,6 +3346,7 @@ struct Ctx32 {
   int jfactor0;                // the same on the finest level
   cudaStream_t st;
   Prof* pr;
+  bool pdl = true;             // launches overlap (not where events time each one)
   int nb = 1;                  // members of a batched ensemble (fields member after member)
   double* const* fold_u = nullptr;   // FP64 state the finest level's last pass adds d to
 };
@@ -3424,13 +3402,13 @@ cudaError_t jacobi_level32(const Ctx32& c, int l, int sweeps, bool zero_init, bo
                            bool fold = false) {
   prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
   cudaError_t e = jacobi32(c.L[l], fold ? sweeps - 1 : sweeps, c.w, zero_init, c.mx->d[l],
-                           c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st, c.pr == nullptr, c.nb, &in_t);
+                           c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st, c.pdl, c.nb, &in_t);
   prof_end(c.pr, PFC_K_LIN_SMOOTH, l, fold ? sweeps - 1 : sweeps, c.st);
   if (fold && e == cudaSuccess) {
     // timed as the correction it replaces
     prof_begin(c.pr, PFC_K_CORRECT, c.st);
     e = jacobi32(c.L[l], 1, c.w, false, c.mx->d[l], c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st,
-                 c.pr == nullptr, c.nb, &in_t, c.fold_u);
+                 c.pdl, c.nb, &in_t, c.fold_u);
     prof_end(c.pr, PFC_K_CORRECT, l, 1, c.st);
   }
   if (in_t)
@@ -3451,14 +3429,14 @@ cudaError_t rb_pass32(const Ctx32& c, int l, int colour, bool zero) {
   const bool pairs = L.n % 4 == 0;              // two cells per thread, float2 moves
   const Launch3 g = launch3(pairs ? L.n / 4 : L.n / 2, L.n, L.n * c.nb);
   if (pairs && zero)                            // a zero start begins with colour 0
-    return launch_k(c.pr == nullptr, k_lin_smooth32_zero, g.grid, g.block, 0, c.st, L, d[0], d[1],
+    return launch_k(c.pdl, k_lin_smooth32_zero, g.grid, g.block, 0, c.st, L, d[0], d[1],
                     d[2], r[0], r[1], r[2], q);
   if (pairs) {
     const March mg = march(L.n, c.nb);
-    return launch_k(c.pr == nullptr, k_lin_smooth32m, mg.grid, mg.block, 0, c.st, L, colour, mg.zc,
+    return launch_k(c.pdl, k_lin_smooth32m, mg.grid, mg.block, 0, c.st, L, colour, mg.zc,
                     d[0], d[1], d[2], r[0], r[1], r[2], q);
   }
-  return launch_k(c.pr == nullptr, zero ? k_lin_smooth32<true> : k_lin_smooth32<false>, g.grid,
+  return launch_k(c.pdl, zero ? k_lin_smooth32<true> : k_lin_smooth32<false>, g.grid,
                   g.block, 0, c.st, L, colour, d[0], d[1], d[2], r[0], r[1], r[2], q);
 }
 
@@ -3468,7 +3446,7 @@ cudaError_t rb_pass32_correct(const Ctx32& c, int l) {
   float* const* d = c.mx->d[l];
   float* const* r = c.mx->r[l];
   const Launch3 g = launch3(L.n / 4, L.n, L.n * c.nb);
-  return launch_k(c.pr == nullptr, k_lin_smooth32_correct, g.grid, g.block, 0, c.st, L,
+  return launch_k(c.pdl, k_lin_smooth32_correct, g.grid, g.block, 0, c.st, L,
                   (const float*)d[0], (const float*)d[1], (const float*)d[2], (const float*)r[0],
                   (const float*)r[1], (const float*)r[2], (const float*)c.mx->q[l], c.fold_u[0],
                   c.fold_u[1], c.fold_u[2]);
@@ -3531,7 +3509,7 @@ cudaError_t launch_prolong_sweep(const Ctx32& c, int l, bool jacobi, bool assign
                   : (assign ? k_lin_prolong_sweep32<TY, TZ, false, true>
                             : k_lin_prolong_sweep32<TY, TZ, false, false>);
   float* const* e = mx.d[l + 1];
-  return launch_k(c.pr == nullptr, k, grid, block, 0, c.st, c.L[l], c.w, (const float*)e[0],
+  return launch_k(c.pdl, k, grid, block, 0, c.st, c.L[l], c.w, (const float*)e[0],
                   (const float*)e[1], (const float*)e[2], mx.d[l][0], mx.d[l][1], mx.d[l][2],
                   mx.t[l][0], mx.t[l][1], mx.t[l][2], (const float*)mx.r[l][0],
                   (const float*)mx.r[l][1], (const float*)mx.r[l][2], (const float*)mx.q[l]);
@@ -3596,7 +3574,7 @@ cudaError_t tail32(const Ctx32& c, int l0, bool zero_init) {
   }
   prof_begin(c.pr, PFC_K_LIN_COARSE, c.st);
   cudaError_t e =
-      launch_k(c.pr == nullptr, k_lin_tail32, dim3(c.nb), dim3(tail_threads(sizes[l0])), smem, c.st, P);
+      launch_k(c.pdl, k_lin_tail32, dim3(c.nb), dim3(tail_threads(sizes[l0])), smem, c.st, P);
   prof_end(c.pr, PFC_K_LIN_COARSE, l0, 1, c.st);
   return e;
 }
@@ -3705,7 +3683,7 @@ cudaError_t ctail32(const Ctx32& c, int l0, bool zero_init, int nd, size_t smem,
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = c.pr == nullptr ? 2 : 1;
+  cfg.numAttrs = c.pdl ? 2 : 1;
   prof_begin(c.pr, PFC_K_LIN_COARSE, c.st);
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_lin_ctail32, P);
   prof_end(c.pr, PFC_K_LIN_COARSE, l0, 1, c.st);
@@ -3793,13 +3771,13 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
                                      : k_lin_restrict_chain32<true, 1>)
                         : (extra > 1 ? k_lin_restrict_chain32<false, 2>
                                      : k_lin_restrict_chain32<false, 1>);
-      e = launch_k(c.pr == nullptr, kern, grid, block, 0, c.st, L, mx.d[l][0], mx.d[l][1],
+      e = launch_k(c.pdl, kern, grid, block, 0, c.st, L, mx.d[l][0], mx.d[l][1],
                    mx.d[l][2], mx.r[l][0], mx.r[l][1], mx.r[l][2], mx.q[l], mx.r[l + 1][0],
                    mx.r[l + 1][1], mx.r[l + 1][2], r2[0], r2[1], r2[2], r3[0], r3[1], r3[2]);
       below = extra;
     } else {
       const Launch3 gr = launch3(nc, nc, nc * c.nb);
-      e = launch_k(c.pr == nullptr,
+      e = launch_k(c.pdl,
                    dzero ? k_lin_residual_restrict32<true> : k_lin_residual_restrict32<false>,
                    gr.grid, gr.block, 0, c.st, L, mx.d[l][0], mx.d[l][1], mx.d[l][2],
                    mx.r[l][0], mx.r[l][1], mx.r[l][2], mx.q[l], mx.r[l + 1][0], mx.r[l + 1][1],
@@ -3825,7 +3803,7 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
   // the colour-0 cells without reading them
   const bool skip0 = c.kind[l] != PFC_SWEEP_JACOBI && c.p->nu2 > 0;
   prof_begin(c.pr, PFC_K_LIN_PROLONG, c.st);
-  e = launch_k(c.pr == nullptr, prolong_kernel(dzero, skip0), prolong_grid(nc, pz, 3 * c.nb),
+  e = launch_k(c.pdl, prolong_kernel(dzero, skip0), prolong_grid(nc, pz, 3 * c.nb),
                dim3(kPrTI * kPrTJ), 0, c.st, L.n, pz, mx.d[l + 1][0], mx.d[l + 1][1],
                mx.d[l + 1][2], mx.d[l][0], mx.d[l][1], mx.d[l][2]);
   prof_end(c.pr, PFC_K_LIN_PROLONG, l, 1, c.st);
@@ -4366,6 +4344,7 @@ cudaError_t mixed_vcycles(MixedBufs& mx, const pfc_params& p, int nl, const int*
   c.nl = nl;
   c.st = st;
   c.pr = pr;
+  c.pdl = !pr || pr->mask == 0;
   c.w = (float)p.jacobi_weight;
   c.jfactor = p.jacobi_factor;
   c.jfactor0 = p.jacobi_factor0;
@@ -4392,12 +4371,12 @@ cudaError_t mixed_vcycles(MixedBufs& mx, const pfc_params& p, int nl, const int*
       const dim3 grid(nc / kChTX, nc / kChTY, (nc / kChTZ) * members),
           block(kChTX, kChTY, kChTZ);
       float* const g2 = extra > 1 ? mx.q[l + 2] : mx.q[l + 1];
-      e = launch_k(pr == nullptr, extra > 1 ? k_restrict_chain32<2> : k_restrict_chain32<1>,
+      e = launch_k(c.pdl, extra > 1 ? k_restrict_chain32<2> : k_restrict_chain32<1>,
                    grid, block, 0, st, sizes[l - 1], (const float*)mx.q[l - 1], mx.q[l],
                    mx.q[l + 1], g2);
     } else {
       const Launch3 g = launch3(nc, nc, nc * members);
-      e = launch_k(pr == nullptr, k_restrict32, g.grid, g.block, 0, st, sizes[l - 1],
+      e = launch_k(c.pdl, k_restrict32, g.grid, g.block, 0, st, sizes[l - 1],
                    (const float*)mx.q[l - 1], mx.q[l]);
     }
     prof_end(pr, PFC_K_RESTRICT, l - 1, 1, st);
@@ -4424,7 +4403,7 @@ cudaError_t mixed_enqueue_correction(const MixedBufs& bufs, const pfc_params& p,
   if (e == cudaSuccess && !folded) {
     prof_begin(pr, PFC_K_CORRECT, st);
     e = launch_correct64(p.n, u[0], u[1], u[2], mx.d[0][0], mx.d[0][1], mx.d[0][2], st,
-                         pr == nullptr, members);
+                         !pr || pr->mask == 0, members);
     prof_end(pr, PFC_K_CORRECT, 0, 1, st);
   }
   return e;
@@ -4439,7 +4418,7 @@ cudaError_t mixed_enqueue_correction(const MixedBufs& bufs, const pfc_params& p,
   if (e == cudaSuccess) {
     prof_begin(pr, PFC_K_CORRECT, st);
     e = launch_correct_df(p.n, u[0], u[1], u[2], mx.d[0][0], mx.d[0][1], mx.d[0][2], st,
-                          pr == nullptr);
+                          !pr || pr->mask == 0);
     prof_end(pr, PFC_K_CORRECT, 0, 1, st);
   }
   return e;

@@ -380,7 +380,6 @@ __device__ __forceinline__ void tail_prolong(const TailParams& P, int l, const T
 // averaged here, the top level's d goes back at the end.
 __global__ void __launch_bounds__(kTailThreads) k_lin_tail32(TailParams P) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float red[2][32];
   __shared__ int done;
   const bool zero_top = P.zero_init != 0;
