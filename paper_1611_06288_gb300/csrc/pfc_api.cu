@@ -374,7 +374,7 @@ cudaError_t enqueue_diagnostics(int n, int members, const double* a, const doubl
   cudaError_t e;
   if (df_fields && lapa)
     e = launch_diagnostics_cached_df(n, as_df(a), as_df(b), as_df(lapa), as_df(lapb), partials,
-                                     dout, st);
+                                     dout, st, pdl);
   else if (df_fields)
     e = launch_diagnostics_df(n, as_df(a), as_df(b), partials, dout, st);
   else if (lapa)
@@ -426,7 +426,7 @@ int enqueue_residual_decide(pfc_ctx* c, const Level64& lv, cudaGraphConditionalH
       S[q] = as_df(lv.S[q]);
     }
     PFC_CUDA(mixed_enqueue_defect(c->mx, lv.L, u, S, as_df(lv.b), c->partials, c->dout, st,
-                                  &c->prof, as_df(c->lap[c->ia])));
+                                  &c->prof, as_df(c->lap[c->ia]), &da, &decided));
   } else if (point) {
     PFC_CUDA(mixed_enqueue_defect_point(c->mx, lv.L, lv.u, lv.S, lv.b, c->lap[c->ib], c->lmu,
                                         c->lom, c->lap[c->ia], c->partials, c->dout, st,
@@ -493,7 +493,7 @@ int enqueue_pre(pfc_ctx* c, const Level64& lv, cudaGraphConditionalHandle h, int
     PFC_TIMED(pr, PFC_K_SOURCE, 0, 1, c->st,
               launch_source_cached_df(lv.L, as_df(lv.b), as_df(c->lap[c->ib]),
                                       as_df(c->lap[c->ic]), as_df(c->S2), as_df(c->S3),
-                                      c->st));
+                                      c->st, c->prof.mask == 0));
   } else {
     PFC_TIMED(pr, PFC_K_SOURCE, 0, 1, c->st,
               launch_source_cached(lv.L, lv.b, c->lap[c->ib], c->lap[c->ic], c->S2, c->S3,
@@ -521,7 +521,7 @@ int enqueue_pre(pfc_ctx* c, const Level64& lv, cudaGraphConditionalHandle h, int
   if (c->M[0]) {
     // M(A phi_*) of this step (Section 5: phi_* = 3/2 phi^k - 1/2 phi^{k-1})
     PFC_CUDA(launch_face_mobility(c->p.n, c->p.mobility_m0, c->p.mobility_m2, lv.b, cprev,
-                                  c->M[0], c->M[1], c->M[2], c->st));
+                                  c->M[0], c->M[1], c->M[2], c->st, c->prof.mask == 0));
     c->prof.launches += 1;
   }
   return enqueue_residual_decide(c, lv, h, use_handle, 1, warm);

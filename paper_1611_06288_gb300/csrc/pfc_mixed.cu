@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(256) k_defect64(Lvl L, const double* __restric
                                                   const double* __restrict__ Mx,
                                                   const double* __restrict__ My,
                                                   const double* __restrict__ Mz) {
+  pdl_wait();
   __shared__ float sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -677,6 +678,7 @@ __global__ void __launch_bounds__(256, 4) k_start64_extrap(
 __global__ void k_face_mobility(int n, double m0, double m2, const double* __restrict__ b,
                                 const double* __restrict__ c, double* __restrict__ Mx,
                                 double* __restrict__ My, double* __restrict__ Mz) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
             k = blockIdx.z;
   if (i >= n || j >= n) return;
@@ -705,6 +707,7 @@ __global__ void __launch_bounds__(256) k_adj_defect64(
     const double* __restrict__ z3, const double* __restrict__ g, const double* __restrict__ a,
     const double* __restrict__ b, float* __restrict__ r1, float* __restrict__ r2,
     float* __restrict__ r3, float* __restrict__ q, double* partials) {
+  pdl_wait();
   __shared__ float sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -743,6 +746,7 @@ __global__ void __launch_bounds__(256) k_adj_accumulate(
     Lvl L, const double* __restrict__ z1, const double* __restrict__ z2,
     const double* __restrict__ z3, const double* __restrict__ a, const double* __restrict__ b,
     double* gk, double* gkm1, double* partials) {
+  pdl_wait();
   __shared__ double sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -820,6 +824,7 @@ __global__ void __launch_bounds__(256, 5) k_defect_df(
     const float2* __restrict__ S2, const float2* __restrict__ S3,
     const float2* __restrict__ b, float* __restrict__ r1, float* __restrict__ r2,
     float* __restrict__ r3, float* __restrict__ q, double* partials, float2* __restrict__ lap) {
+  pdl_wait();
   __shared__ float sm[32];
   const int n = L.n;
   const int cells = n * n * n;
@@ -961,6 +966,7 @@ __global__ void k_diagnostics_df(int n, const float2* __restrict__ a,
 
 // Fixed-order df sum of the block partials -> out[0..5] as doubles.
 __global__ void k_reduce_df6(const float2* __restrict__ partials, int nparts, double* out) {
+  pdl_wait();
   __shared__ float2 sm[32 * 6];
   df acc[6];
 #pragma unroll
@@ -1037,6 +1043,7 @@ __global__ void k_source_cached_df(LvlD L, const float2* __restrict__ b,
                                    const float2* __restrict__ lapb,
                                    const float2* __restrict__ lapc, float2* __restrict__ S2,
                                    float2* __restrict__ S3) {
+  pdl_wait();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)L.n * L.n * L.n) return;
   const int u = (int)t;
@@ -1052,6 +1059,7 @@ __global__ void k_diagnostics_cached_df(int n, const float2* __restrict__ a,
                                         const float2* __restrict__ b,
                                         const float2* __restrict__ lapa,
                                         const float2* __restrict__ lapb, float2* partials) {
+  pdl_wait();
   __shared__ float2 sm[32 * 6];
   const int cells = n * n * n;
   df acc[6];
@@ -3900,14 +3908,11 @@ cudaError_t launch_defect64(const Lvl& L, const double* phi, const double* mu,
   const int64_t need = ((int64_t)L.n * L.n * L.n + kReduceThreads - 1) / kReduceThreads;
   if (nbx > need) nbx = (int)need;
   if (nbx < 1) nbx = 1;
-  if (Mx)
-    k_defect64<true><<<dim3(nbx, members), kReduceThreads, 0, st>>>(
-        L, phi, mu, om, S1, S2, S3, b, r1, r2, r3, q, partials, lap, c1m, Mx, My, Mz);
-  else
-    k_defect64<false><<<dim3(nbx, members), kReduceThreads, 0, st>>>(
-        L, phi, mu, om, S1, S2, S3, b, r1, r2, r3, q, partials, lap, c1m, Mx, My, Mz);
-  k_reduce1<<<members, kReduceThreads, 0, st>>>(partials, nbx, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_ex(pdl, Mx ? k_defect64<true> : k_defect64<false>, dim3(nbx, members),
+                            dim3(kReduceThreads), 0, st, L, phi, mu, om, S1, S2, S3, b, r1, r2, r3,
+                            q, partials, lap, c1m, Mx, My, Mz);
+  if (e == cudaSuccess) e = launch_reduce1(pdl, partials, nbx, out, members, st, da, decided);
+  return e;
 }
 
 cudaError_t launch_defect64_point(const Lvl& L, const double* b, const double* mu,
@@ -3969,10 +3974,9 @@ cudaError_t launch_start64_extrap(const Lvl& L, const double* b, const double* c
 }
 
 cudaError_t launch_face_mobility(int n, double m0, double m2, const double* b, const double* c,
-                                 double* Mx, double* My, double* Mz, cudaStream_t st) {
+                                 double* Mx, double* My, double* Mz, cudaStream_t st, bool pdl) {
   const Launch3 g = launch3(n, n, n);
-  k_face_mobility<<<g.grid, g.block, 0, st>>>(n, m0, m2, b, c, Mx, My, Mz);
-  return cudaGetLastError();
+  return launch_k(pdl, k_face_mobility, g.grid, g.block, 0, st, n, m0, m2, b, c, Mx, My, Mz);
 }
 
 cudaError_t launch_correct64(int n, double* u1, double* u2, double* u3, const float* d1,
@@ -3987,10 +3991,10 @@ cudaError_t launch_adj_defect64(const Lvl& L, const double* z1, const double* z2
                                 const double* b, float* r1, float* r2, float* r3, float* q,
                                 double* partials, double* out, cudaStream_t st) {
   const int nb = wave_blocks(k_adj_defect64, (int64_t)L.n * L.n * L.n);
-  k_adj_defect64<<<nb, kReduceThreads, 0, st>>>(L, z1, z2, z3, g, a, b, r1, r2, r3, q,
-                                                partials);
-  k_reduce1<<<1, kReduceThreads, 0, st>>>(partials, nb, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_ex(true, k_adj_defect64, dim3(nb), dim3(kReduceThreads), 0, st, L, z1, z2,
+                            z3, g, a, b, r1, r2, r3, q, partials);
+  if (e == cudaSuccess) e = launch_reduce1(true, partials, nb, out, 1, st, nullptr, nullptr);
+  return e;
 }
 
 cudaError_t launch_adj_accumulate(const Lvl& L, const double* z1, const double* z2,
@@ -3998,21 +4002,22 @@ cudaError_t launch_adj_accumulate(const Lvl& L, const double* z1, const double* 
                                   double* gk, double* gkm1, double* partials, double* out,
                                   cudaStream_t st) {
   const int nb = wave_blocks(k_adj_accumulate, (int64_t)L.n * L.n * L.n);
-  k_adj_accumulate<<<nb, kReduceThreads, 0, st>>>(L, z1, z2, z3, a, b, gk, gkm1, partials);
-  k_reduce1<<<1, kReduceThreads, 0, st>>>(partials, nb, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_ex(true, k_adj_accumulate, dim3(nb), dim3(kReduceThreads), 0, st, L, z1,
+                            z2, z3, a, b, gk, gkm1, partials);
+  if (e == cudaSuccess) e = launch_reduce1(true, partials, nb, out, 1, st, nullptr, nullptr);
+  return e;
 }
 
 cudaError_t launch_defect_df(const Lvl& L, const float2* phi, const float2* mu,
                              const float2* om, const float2* S1, const float2* S2,
                              const float2* S3, const float2* b, float* r1, float* r2, float* r3,
                              float* q, double* partials, double* out, cudaStream_t st,
-                             float2* lap) {
+                             float2* lap, bool pdl, const DecideArgs* da, bool* decided) {
   const int nb = wave_blocks(k_defect_df, (int64_t)L.n * L.n * L.n);
-  k_defect_df<<<nb, kReduceThreads, 0, st>>>(to_df(L), phi, mu, om, S1, S2, S3, b, r1, r2, r3,
-                                             q, partials, lap);
-  k_reduce1<<<1, kReduceThreads, 0, st>>>(partials, nb, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_ex(pdl, k_defect_df, dim3(nb), dim3(kReduceThreads), 0, st, to_df(L), phi,
+                            mu, om, S1, S2, S3, b, r1, r2, r3, q, partials, lap);
+  if (e == cudaSuccess) e = launch_reduce1(pdl, partials, nb, out, 1, st, da, decided);
+  return e;
 }
 
 cudaError_t launch_source_df(const Lvl& L, const float2* b, const float2* c, float2* S2,
@@ -4060,20 +4065,24 @@ cudaError_t launch_laplacian_df(int n, const float2* v, float2* lap, cudaStream_
 }
 
 cudaError_t launch_source_cached_df(const Lvl& L, const float2* b, const float2* lapb,
-                                    const float2* lapc, float2* S2, float2* S3, cudaStream_t st) {
-  k_source_cached_df<<<grid_for((int64_t)L.n * L.n * L.n), kThreads, 0, st>>>(to_df(L), b, lapb,
-                                                                              lapc, S2, S3);
-  return cudaGetLastError();
+                                    const float2* lapc, float2* S2, float2* S3, cudaStream_t st,
+                                    bool pdl) {
+  return launch_ex(pdl, k_source_cached_df, dim3(grid_for((int64_t)L.n * L.n * L.n)),
+                   dim3(kThreads), 0, st, to_df(L), b, lapb, lapc, S2, S3);
 }
 
 cudaError_t launch_diagnostics_cached_df(int n, const float2* a, const float2* b,
                                          const float2* lapa, const float2* lapb,
-                                         double* partials, double* out, cudaStream_t st) {
+                                         double* partials, double* out, cudaStream_t st,
+                                         bool pdl) {
   const int nb = wave_blocks(k_diagnostics_cached_df, (int64_t)n * n * n);
   float2* parts = reinterpret_cast<float2*>(partials);
-  k_diagnostics_cached_df<<<nb, kReduceThreads, 0, st>>>(n, a, b, lapa, lapb, parts);
-  k_reduce_df6<<<1, kReduceThreads, 0, st>>>(parts, nb, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_ex(pdl, k_diagnostics_cached_df, dim3(nb), dim3(kReduceThreads), 0, st, n,
+                            a, b, lapa, lapb, parts);
+  if (e == cudaSuccess)
+    e = launch_ex(pdl, k_reduce_df6, dim3(1), dim3(kReduceThreads), 0, st, (const float2*)parts, nb,
+                  out);
+  return e;
 }
 
 cudaError_t launch_df_from_f64(int64_t count, const double* x, float2* y, cudaStream_t st) {
@@ -4316,10 +4325,12 @@ cudaError_t mixed_enqueue_start_extrap(MixedBufs& mx, const Lvl& L0, double* con
 
 cudaError_t mixed_enqueue_defect(MixedBufs& mx, const Lvl& L0, float2* const u[3],
                                  float2* const S[3], const float2* b, double* partials,
-                                 double* dout, cudaStream_t st, Prof* pr, float2* lap) {
+                                 double* dout, cudaStream_t st, Prof* pr, float2* lap,
+                                 const DecideArgs* da, bool* decided) {
   prof_begin(pr, PFC_K_DEFECT, st);
   cudaError_t e = launch_defect_df(L0, u[0], u[1], u[2], S[0], S[1], S[2], b, mx.r[0][0],
-                                   mx.r[0][1], mx.r[0][2], mx.q[0], partials, dout, st, lap);
+                                   mx.r[0][1], mx.r[0][2], mx.q[0], partials, dout, st, lap,
+                                   !pr || pr->mask == 0, da, decided);
   prof_end(pr, PFC_K_DEFECT, 0, 2, st);
   return e;
 }

@@ -110,7 +110,8 @@ cudaError_t mixed_enqueue_start_extrap(MixedBufs& mx, const Lvl& L0, double* con
 // sum of |r|^2 at dout[0] (two launches).  S[0] is S1 (= b in a time step).
 cudaError_t mixed_enqueue_defect(MixedBufs& mx, const Lvl& L0, float2* const u[3],
                                  float2* const S[3], const float2* b, double* partials,
-                                 double* dout, cudaStream_t st, Prof* pr, float2* lap);
+                                 double* dout, cudaStream_t st, Prof* pr, float2* lap,
+                                 const DecideArgs* da = nullptr, bool* decided = nullptr);
 
 // One defect correction after mixed_enqueue_defect: q restricted to every
 // level, p.inner_cycles FP32 V-cycles on J d = r from d = 0, then u += d in
@@ -146,10 +147,12 @@ cudaError_t launch_widen_f64(int64_t count, const float* x, double* y, cudaStrea
 // launch_diagnostics_cached.
 cudaError_t launch_laplacian_df(int n, const float2* v, float2* lap, cudaStream_t st);
 cudaError_t launch_source_cached_df(const Lvl& L, const float2* b, const float2* lapb,
-                                    const float2* lapc, float2* S2, float2* S3, cudaStream_t st);
+                                    const float2* lapc, float2* S2, float2* S3, cudaStream_t st,
+                                    bool pdl = false);
 cudaError_t launch_diagnostics_cached_df(int n, const float2* a, const float2* b,
                                          const float2* lapa, const float2* lapb,
-                                         double* partials, double* out, cudaStream_t st);
+                                         double* partials, double* out, cudaStream_t st,
+                                         bool pdl = false);
 
 // Whole-field conversions FP64 <-> df (count cells; in place allowed).
 cudaError_t launch_df_from_f64(int64_t count, const double* x, float2* y, cudaStream_t st);
@@ -195,7 +198,8 @@ cudaError_t launch_start64_extrap(const Lvl& L, const double* b, const double* c
 // Face mobilities M(A phi_*), phi_* = 3/2 b - 1/2 c, M(phi) = m0 + m2 phi^2,
 // face i+1/2 of each axis stored at cell i (FP64).
 cudaError_t launch_face_mobility(int n, double m0, double m2, const double* b, const double* c,
-                                 double* Mx, double* My, double* Mz, cudaStream_t st);
+                                 double* Mx, double* My, double* Mz, cudaStream_t st,
+                                 bool pdl = false);
 cudaError_t launch_correct64(int n, double* u1, double* u2, double* u3, const float* d1,
                              const float* d2, const float* d3, cudaStream_t st,
                              bool pdl = true, int members = 1);
@@ -203,7 +207,8 @@ cudaError_t launch_defect_df(const Lvl& L, const float2* phi, const float2* mu,
                              const float2* om, const float2* S1, const float2* S2,
                              const float2* S3, const float2* b, float* r1, float* r2, float* r3,
                              float* q, double* partials, double* out, cudaStream_t st,
-                             float2* lap = nullptr);
+                             float2* lap = nullptr, bool pdl = false,
+                             const DecideArgs* da = nullptr, bool* decided = nullptr);
 cudaError_t launch_lin_residual_restrict32(const Lvl& L, bool zero, const float* d1,
                                           const float* d2, const float* d3, const float* r1,
                                           const float* r2, const float* r3, const float* q,
