@@ -87,9 +87,8 @@ NCU_TRAFFIC = {("mixed", "defect", 128): 150.8e6,   # profiles/k_defect64_fx_128
 # FP64-ALU-bound kernel classes of a precision: FP64 flops per cell of one
 # counted launch (FMA = 2) and launches per group.  The full FP64 defect forms
 # the three Laplacians' neighbour sums in exact int64 fixed point (no FP64
-# flops) and its rows in 6 DFMA + 4 DADD + 2 DMUL per cell (ncu: DFMA, DADD
-# and DMUL thread-instruction rates 3:2:1): 18 flops.
-KERNEL_FLOPS = {("mixed", "defect"): (18.0, 2)}
+# flops) and its rows in 6 DFMA + 4 DADD + 1 DMUL per cell: 17 flops.
+KERNEL_FLOPS = {("mixed", "defect"): (17.0, 2)}
 
 # Algorithmic bytes per cell of the FP64 defect class (the ALU-bound class
 # above), reported beside its FP64 roofline: a full defect reads phi, mu, om,

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "pfc.h"
+#include "pfc_fixed.cuh"
 
 namespace pfc {
 
@@ -77,7 +78,7 @@ __device__ __forceinline__ T nbsum_coherent(const T* v, const Stencil& s) {
 
 // Cubic term f(a) = (a+b)(a^2+b^2)/4 of Eq. 5.2.
 __device__ __forceinline__ double cubic_f(double a, double b) {
-  return 0.25 * (a + b) * fma(a, a, b * b);
+  return fix_quarter(a + b) * fma(a, a, b * b);
 }
 
 // r = S - N(u) at one cell (Eqs. 5.4-5.6 with M = 1); lap receives the

@@ -300,8 +300,9 @@ constexpr int kFxTX = 32, kFxTY = 8;
 constexpr int kFxRing = 4;
 constexpr size_t kFxSmem = (size_t)kFxRing * 3 * (kFxTY + 2) * (kFxTX + 2) * sizeof(int64_t);
 
-// The three rows at one cell from the unscaled Laplacians, in 12 FP64
-// operations: x = S1 - phi + tau/h^2 Lap mu, y = S2 - mu + f + c1 phi +
+// The three rows at one cell from the unscaled Laplacians, in 11 FP64
+// operations and an exact quarter on the integer pipe (as a twelfth operation
+// it cost 3 us of 73 at 128^3 and 23 of 486 at 256^3): x = S1 - phi + tau/h^2 Lap mu, y = S2 - mu + f + c1 phi +
 // 1/h^2 Lap om with f = (phi + b)(phi^2 + b^2)/4 (Eq. 5.2), z = S3 - om +
 // 1/(2h^2) Lap phi, each rounded to FP32 on the integer pipe.  The Newton
 // coefficient q = f'(phi) + c1 only feeds the FP32 preconditioner: it is
@@ -314,7 +315,7 @@ __device__ __forceinline__ void defect_rows(const Lvl& L, double c1, float c1f, 
   const double t = p + bb;
   const double sq = fma(p, p, bb * bb);
   const double x = fma(L.tg, lmu, s1 - p);
-  const double y = fma(L.g, lom, fma(c1, p, fma(0.25 * t, sq, s2 - mm)));
+  const double y = fma(L.g, lom, fma(c1, p, fma(fix_quarter(t), sq, s2 - mm)));
   const double z = fma(L.gh, lphi, s3 - w);
   xf = d2f_rn(x);
   yf = d2f_rn(y);
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(256, 4) k_start64_extrap(
     lapom1[t] = lo;
     const double sq = fma(p, p, vb * vb);
     const double x = fma(L.tg, lm, cmb);
-    const double y = fma(L.g, a, fma(c1, bs, fma(0.25 * bs, sq, -mm)));
+    const double y = fma(L.g, a, fma(c1, bs, fma(fix_quarter(bs), sq, -mm)));
     const double z = fma(L.gh, k3, -w);
     const float xf = d2f_rn(x), yf = d2f_rn(y), zf = d2f_rn(z);
     const float pf = d2f_rn(p), bf = d2f_rn(vb);
