@@ -1738,6 +1738,57 @@ __global__ void k_lin_residual_restrict32(LvlF L, const float* __restrict__ d1,
   (c3 + offc)[ci] = 0.125f * a[2];
 }
 
+// The same on a level of few cells, three threads a coarse cell: each forms the
+// sums of one field over r and d (and the first one that of q d_phi), they meet
+// in shared memory, and thread f ends row f.  Every sum keeps its order, so the
+// bits are those of one thread for all three, whose 128 loads come in several
+// rounds that so few threads do not hide.  us, one thread / three: 10^3 coarse
+// cells 5.2 / 4.2, 12^3 5.5 / 4.2, 20^3 5.8 / 4.4, 24^3 5.8 / 4.6; but 40^3
+// 7.2 / 8.2, 48^3 8.6 / 10.3, 39 x 12^3 7.1 / 7.2, 128^3 99 / 152.
+constexpr int kRrSmall = 1 << 14;      // coarse cells at most
+constexpr int kRrCells = 64;           // of a block, at most
+
+__global__ void __launch_bounds__(3 * kRrCells) k_lin_residual_restrict32s(
+    LvlF L, const float* __restrict__ d1, const float* __restrict__ d2,
+    const float* __restrict__ d3, const float* __restrict__ r1, const float* __restrict__ r2,
+    const float* __restrict__ r3, const float* __restrict__ q, float* __restrict__ c1,
+    float* __restrict__ c2, float* __restrict__ c3) {
+  pdl_wait();
+  __shared__ float laps[3][kRrCells], qps[kRrCells];
+  const int n = L.n, nc = n >> 1, f = threadIdx.z, t = threadIdx.y * blockDim.x + threadIdx.x;
+  const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
+  int K = blockIdx.z;
+  const int m = member_of(K, nc);
+  const bool on = I < nc && J < nc;
+  const size_t off = (size_t)m * n * n * n, offc = (size_t)m * nc * nc * nc;
+  float rsum = 0.f, own = 0.f;
+  if (on) {
+    int in[8], out[24];
+    block_indices(I, J, K, n, in, out);
+    const float* const r = (f == 0 ? r1 : f == 1 ? r2 : r3) + off;
+    const float* const d = (f == 0 ? d1 : f == 1 ? d2 : d3) + off;
+    float v[8], so = 0.f, qp = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) rsum += __ldg(r + in[c]);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) own += v[c] = __ldg(d + in[c]);
+#pragma unroll
+    for (int c = 0; c < 24; ++c) so += __ldg(d + out[c]);
+    laps[f][t] = fmaf(-3.f, own, so);
+    if (f == 0) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) qp = fmaf(__ldg(q + off + in[c]), v[c], qp);
+      qps[t] = qp;
+    }
+  }
+  __syncthreads();
+  if (!on) return;
+  // row f: own d_f, the field under the Laplacian (d_mu, d_om, d_phi)
+  float a = fmaf(f == 0 ? L.tg : f == 1 ? L.g : L.gh, laps[f == 2 ? 0 : f + 1][t], rsum - own);
+  if (f == 1) a += qps[t];
+  (f == 0 ? c1 : f == 1 ? c2 : c3)[offc + split_index(I, J, K, nc)] = 0.125f * a;
+}
+
 // The restriction of k_lin_residual_restrict32 followed by EXTRA more
 // levels of plain 8-cell averages, in one launch.  Without pre-smoothing
 // (nu1 = 0) every coarser level starts its V-cycle from d = 0, so its own
@@ -3708,6 +3759,23 @@ bool block_tail_at(const Ctx32& c, int l) {
   return tail_smem_bytes(sizes, l, c.nl) <= kTailMaxSmem;
 }
 
+// rho = r - J d (r where zero: d = 0) averaged onto the next level.
+cudaError_t launch_lin_restrict(bool pdl, const LvlF& L, bool zero, int members, const float* d1,
+                                const float* d2, const float* d3, const float* r1,
+                                const float* r2, const float* r3, const float* q, float* c1,
+                                float* c2, float* c3, cudaStream_t st) {
+  const int nc = L.n / 2;
+  if (!zero && (int64_t)nc * nc * nc * members <= kRrSmall) {
+    const int bx = nc < 32 ? nc : 32, by = kRrCells / bx < nc ? kRrCells / bx : nc;
+    return launch_k(pdl, k_lin_residual_restrict32s,
+                    dim3((nc + bx - 1) / bx, (nc + by - 1) / by, nc * members), dim3(bx, by, 3), 0,
+                    st, L, d1, d2, d3, r1, r2, r3, q, c1, c2, c3);
+  }
+  const Launch3 g = launch3(nc, nc, nc * members);
+  return launch_k(pdl, zero ? k_lin_residual_restrict32<true> : k_lin_residual_restrict32<false>,
+                  g.grid, g.block, 0, st, L, d1, d2, d3, r1, r2, r3, q, c1, c2, c3);
+}
+
 // Whether vcycle32 at level l restricts to l + 1 with a launch of its own
 // (not the cluster tail, the shared-memory tail or the coarsest solve).
 bool restricts_alone(const Ctx32& c, int l) {
@@ -3785,12 +3853,9 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
                    mx.r[l + 1][1], mx.r[l + 1][2], r2[0], r2[1], r2[2], r3[0], r3[1], r3[2]);
       below = extra;
     } else {
-      const Launch3 gr = launch3(nc, nc, nc * c.nb);
-      e = launch_k(c.pdl,
-                   dzero ? k_lin_residual_restrict32<true> : k_lin_residual_restrict32<false>,
-                   gr.grid, gr.block, 0, c.st, L, mx.d[l][0], mx.d[l][1], mx.d[l][2],
-                   mx.r[l][0], mx.r[l][1], mx.r[l][2], mx.q[l], mx.r[l + 1][0], mx.r[l + 1][1],
-                   mx.r[l + 1][2]);
+      e = launch_lin_restrict(c.pdl, L, dzero, c.nb, mx.d[l][0], mx.d[l][1], mx.d[l][2],
+                              mx.r[l][0], mx.r[l][1], mx.r[l][2], mx.q[l], mx.r[l + 1][0],
+                              mx.r[l + 1][1], mx.r[l + 1][2], c.st);
     }
     prof_end(c.pr, PFC_K_LIN_RESTRICT, l, 1, c.st);
   }
@@ -4102,11 +4167,7 @@ cudaError_t launch_lin_residual_restrict32(const Lvl& L, bool zero, const float*
                                           const float* d2, const float* d3, const float* r1,
                                           const float* r2, const float* r3, const float* q,
                                           float* c1, float* c2, float* c3, cudaStream_t st) {
-  const int nc = L.n / 2;
-  const Launch3 g = launch3(nc, nc, nc);
-  return launch_k(true,
-                  zero ? k_lin_residual_restrict32<true> : k_lin_residual_restrict32<false>,
-                  g.grid, g.block, 0, st, to_f32(L), d1, d2, d3, r1, r2, r3, q, c1, c2, c3);
+  return launch_lin_restrict(true, to_f32(L), zero, 1, d1, d2, d3, r1, r2, r3, q, c1, c2, c3, st);
 }
 
 cudaError_t launch_lin_restrict_chain32(const Lvl& L, bool zero, int extra, const float* d1,
