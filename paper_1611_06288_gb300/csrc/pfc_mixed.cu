@@ -2866,6 +2866,7 @@ __device__ void tail_vcycle(float* smem, const TailParams& P, bool zero_top, flo
 }
 
 #include "pfc_tail.cuh"
+#include "pfc_jacobi2.cuh"
 
 // Shared memory of the tail starting at level l0.
 size_t tail_smem_bytes(const int* sizes, int l0, int nl) {
@@ -3413,10 +3414,11 @@ struct Ctx32 {
 
 // `sweeps` damped Jacobi sweeps d -> t -> d ...; *in_t: whether the iterate is
 // in t, on entry and on return.  u (n % 4 == 0, not for the sweep from zero):
-// the last sweep adds to u instead.
+// the last sweep adds to u instead.  *launches (may be null): their number.
 cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* const* d,
                      float* const* t, float* const* r, const float* q, cudaStream_t st,
-                     bool pdl, int nb, bool* in_t, double* const* u = nullptr) {
+                     bool pdl, int nb, bool* in_t, double* const* u = nullptr,
+                     int* launches = nullptr) {
   const int n = L.n;
   const bool pairs = n % 4 == 0;                // two cells per thread, float2 moves
   const Launch3 g = launch3(pairs ? n / 2 : n, n, n * nb);
@@ -3428,11 +3430,17 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
       src[c] = t[c];
       dst[c] = d[c];
     }
-  int done = 0;
+  const bool twice = jacobi2_pays(n, nb, d, t, r, q);
+  int done = 0, count = 0;
   cudaError_t e = cudaSuccess;
   while (done < sweeps && e == cudaSuccess) {
     const bool z = zero_init && done == 0;
-    if (pairs && z)
+    const bool two = twice && sweeps - done >= (u ? 3 : 2);     // the sweep into u alone
+    if (two && z)
+      e = launch_jacobi2<true>(L, w, src, dst, r, q, st, pdl, nb);
+    else if (two)
+      e = launch_jacobi2<false>(L, w, src, dst, r, q, st, pdl, nb);
+    else if (pairs && z)
       e = launch_k(pdl, k_lin_jacobi32_zero, g.grid, g.block, 0, st, L, w, dst[0], dst[1], dst[2],
                    r[0], r[1], r[2], q);
     else if (u && done + 1 == sweeps)
@@ -3444,7 +3452,8 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
     else
       e = launch_k(pdl, z ? k_lin_jacobi32<true> : k_lin_jacobi32<false>, g.grid, g.block, 0,
                    st, L, w, src[0], src[1], src[2], dst[0], dst[1], dst[2], r[0], r[1], r[2], q);
-    done += 1;
+    done += two ? 2 : 1;
+    count += 1;
     for (int c = 0; c < 3; ++c) {
       float* x = src[c];
       src[c] = dst[c];
@@ -3452,6 +3461,7 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
     }
   }
   *in_t = src[0] != d[0];
+  if (launches) *launches = count;
   return e;
 }
 
@@ -3460,15 +3470,19 @@ cudaError_t jacobi32(const LvlF& L, int sweeps, float w, bool zero_init, float* 
 // the last sweep adds to c.fold_u (n % 4 == 0).
 cudaError_t jacobi_level32(const Ctx32& c, int l, int sweeps, bool zero_init, bool in_t,
                            bool fold = false) {
+  float* const* d = c.mx->d[l];
+  float* const* t = c.mx->t[l];
+  float* const* r = c.mx->r[l];
+  const float* q = c.mx->q[l];
+  int launches = 0;
   prof_begin(c.pr, PFC_K_LIN_SMOOTH, c.st);
-  cudaError_t e = jacobi32(c.L[l], fold ? sweeps - 1 : sweeps, c.w, zero_init, c.mx->d[l],
-                           c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st, c.pdl, c.nb, &in_t);
-  prof_end(c.pr, PFC_K_LIN_SMOOTH, l, fold ? sweeps - 1 : sweeps, c.st);
+  cudaError_t e = jacobi32(c.L[l], fold ? sweeps - 1 : sweeps, c.w, zero_init, d, t, r, q, c.st, c.pdl, c.nb,
+                           &in_t, nullptr, &launches);
+  prof_end(c.pr, PFC_K_LIN_SMOOTH, l, launches, c.st);
   if (fold && e == cudaSuccess) {
     // timed as the correction it replaces
     prof_begin(c.pr, PFC_K_CORRECT, c.st);
-    e = jacobi32(c.L[l], 1, c.w, false, c.mx->d[l], c.mx->t[l], c.mx->r[l], c.mx->q[l], c.st,
-                 c.pdl, c.nb, &in_t, c.fold_u);
+    e = jacobi32(c.L[l], 1, c.w, false, d, t, r, q, c.st, c.pdl, c.nb, &in_t, c.fold_u);
     prof_end(c.pr, PFC_K_CORRECT, l, 1, c.st);
   }
   if (in_t)
