@@ -274,14 +274,14 @@ __global__ void __launch_bounds__(256) k_defect64(Lvl L, const double* __restric
 // FP64 residual up to rounding order (the Laplacians: exact sums of the
 // quantised inputs and one rounding, instead of five FP64 roundings).
 //
-// Tiling: a block of kFxTX x kFxTY threads owns that column of cells over
+// Tiling: a block of kFxTX x TY threads owns that column of cells over
 // `zc` planes starting at plane k0 and marches upwards in z.  Each thread
 // keeps the fixed-point images of its cell in the planes k-1, k, k+1 in
 // registers; the images of plane k, with a one-cell halo in x and y (wrapped
 // periodically), sit in shared memory for the four in-plane neighbours.  So
 // every value is loaded and converted once per block (plus the halo), not
 // once per neighbour, and the raw values of the next plane are loaded one
-// plane ahead.  Threads past the grid edge (n < kFxTX or n < kFxTY) load
+// plane ahead.  Threads past the grid edge (n < kFxTX or n < TY) load
 // wrapped cells to fill the tile and write nothing.
 //
 // lap (may be null) receives the unscaled Laplacian of phi, lapmu and lapom
@@ -293,19 +293,26 @@ __global__ void __launch_bounds__(256) k_defect64(Lvl L, const double* __restric
 // Laplacians in FP64 from global memory (a block vote per plane); a cell
 // whose own value in the plane above is out of range does so alone.  Same
 // outputs either way.  Per-block partial sums of |r|^2 as k_defect64.
-constexpr int kFxTX = 32, kFxTY = 8;
+//
+// TY = 4, eight blocks an SM: 128^3 66.6 us, 256^3 446, 96^3 32.5; TY = 8, four
+// blocks, 69.8, 463, 33.0 (more warps wait at a barrier; 64 x 4 cells 70.9, 472,
+// 42; 32 x 16, two blocks, 72.8, 492, 33.6).  TY = 8 stays for ensembles whose
+// columns of four rows are more than the partial-sum slots.
+constexpr int kFxTX = 32;
 // Shared-memory ring of the fixed-point images of planes k-1, k, k+1 (own
 // cells, and the halo of plane k): four slots, so one barrier per plane
 // orders every write after the reads of the slot's previous plane.
 constexpr int kFxRing = 4;
-constexpr size_t kFxSmem = (size_t)kFxRing * 3 * (kFxTY + 2) * (kFxTX + 2) * sizeof(int64_t);
+template <int TY>
+constexpr size_t kFxSmem = (size_t)kFxRing * 3 * (TY + 2) * (kFxTX + 2) * sizeof(int64_t);
 
 // The three rows at one cell from the unscaled Laplacians, in 11 FP64
 // operations and an exact quarter on the integer pipe (as a twelfth operation
-// it cost 3 us of 73 at 128^3 and 23 of 486 at 256^3): x = S1 - phi + tau/h^2 Lap mu, y = S2 - mu + f + c1 phi +
-// 1/h^2 Lap om with f = (phi + b)(phi^2 + b^2)/4 (Eq. 5.2), z = S3 - om +
-// 1/(2h^2) Lap phi, each rounded to FP32 on the integer pipe.  The Newton
-// coefficient q = f'(phi) + c1 only feeds the FP32 preconditioner: it is
+// it cost 3 us of 73 at 128^3 and 23 of 486 at 256^3):
+// x = S1 - phi + tau/h^2 Lap mu, y = S2 - mu + f + c1 phi + 1/h^2 Lap om with
+// f = (phi + b)(phi^2 + b^2)/4 (Eq. 5.2), z = S3 - om + 1/(2h^2) Lap phi, each
+// rounded to FP32 on the integer pipe.  The Newton coefficient q = f'(phi) + c1
+// only feeds the FP32 preconditioner: it is
 // formed in FP32 from phi and b rounded to FP32 (a few FP32 roundings).
 __device__ __forceinline__ void defect_rows(const Lvl& L, double c1, float c1f, double p,
                                             double mm, double w, double bb, double lmu,
@@ -324,7 +331,8 @@ __device__ __forceinline__ void defect_rows(const Lvl& L, double c1, float c1f, 
   qf = fmaf(0.75f * pf, pf, fmaf(0.5f * pf, bf, fmaf(0.25f * bf, bf, c1f)));
 }
 
-__global__ void __launch_bounds__(kFxTX * kFxTY, 4) k_defect64_fx(
+template <int TY>
+__global__ void __launch_bounds__(kFxTX * TY, 32 / TY) k_defect64_fx(
     Lvl L, int zc, const double* __restrict__ phi, const double* __restrict__ mu,
     const double* __restrict__ om, const double* __restrict__ S1, const double* __restrict__ S2,
     const double* __restrict__ S3, const double* __restrict__ b, float* __restrict__ r1,
@@ -332,9 +340,9 @@ __global__ void __launch_bounds__(kFxTX * kFxTY, 4) k_defect64_fx(
     double* __restrict__ lap, const double* __restrict__ c1m, double* __restrict__ lapmu,
     double* __restrict__ lapom) {
   pdl_wait();
-  extern __shared__ int64_t ring[];   // [kFxRing][3][kFxTY + 2][kFxTX + 2]
+  extern __shared__ int64_t ring[];   // [kFxRing][3][TY + 2][kFxTX + 2]
   __shared__ float sm[32];
-  constexpr int TW = kFxTX + 2, TP = (kFxTY + 2) * TW, TS = 3 * TP;
+  constexpr int TW = kFxTX + 2, TP = (TY + 2) * TW, TS = 3 * TP;
   const int n = L.n, nn = n * n;
   const int chunks = (n + zc - 1) / zc;
   int zb = blockIdx.z;
@@ -346,23 +354,23 @@ __global__ void __launch_bounds__(kFxTX * kFxTY, 4) k_defect64_fx(
   const double c1 = c1m ? c1m[m] : L.c1;
   const float c1f = d2f_rn(c1);
   const int tid = threadIdx.x, tx = tid % kFxTX, ty = tid / kFxTX;   // 1-D block
-  const int i0 = blockIdx.x * kFxTX, j0 = blockIdx.y * kFxTY;
+  const int i0 = blockIdx.x * kFxTX, j0 = blockIdx.y * TY;
   const int k0 = zb * zc, k1 = min(n, k0 + zc);
   const bool active = i0 + tx < n && j0 + ty < n;
   const int iw = (i0 + tx) % n, jw = (j0 + ty) % n;     // wrapped own column
   const int own = jw * n + iw;
   const int ocell = (ty + 1) * TW + tx + 1;              // own cell in a tile plane
-  // halo cell of this thread (tid < 2 kFxTY + 2 kFxTX): in-plane index and
+  // halo cell of this thread (tid < 2 TY + 2 kFxTX): in-plane index and
   // tile position
   int hidx = -1, hcell = 0;
-  if (tid < 2 * kFxTY) {
-    const int r = tid % kFxTY, side = tid / kFxTY;        // x = i0 - 1 or i0 + kFxTX
+  if (tid < 2 * TY) {
+    const int r = tid % TY, side = tid / TY;        // x = i0 - 1 or i0 + kFxTX
     hcell = (r + 1) * TW + (side ? kFxTX + 1 : 0);
     hidx = ((j0 + r) % n) * n + (side ? (i0 + kFxTX) % n : (i0 - 1 + n) % n);
-  } else if (tid < 2 * kFxTY + 2 * kFxTX) {
-    const int h = tid - 2 * kFxTY, c = h % kFxTX, side = h / kFxTX;   // y = j0 - 1 or j0 + kFxTY
-    hcell = (side ? kFxTY + 1 : 0) * TW + c + 1;
-    hidx = (side ? (j0 + kFxTY) % n : (j0 - 1 + n) % n) * n + (i0 + c) % n;
+  } else if (tid < 2 * TY + 2 * kFxTX) {
+    const int h = tid - 2 * TY, c = h % kFxTX, side = h / kFxTX;   // y = j0 - 1 or j0 + TY
+    hcell = (side ? TY + 1 : 0) * TW + c + 1;
+    hidx = (side ? (j0 + TY) % n : (j0 - 1 + n) % n) * n + (i0 + c) % n;
   }
 #define PFC_FX_FLD(f) ((f) == 0 ? phi : (f) == 1 ? mu : om)
   // Software pipeline over the planes: the images of plane k+1 (own cells)
@@ -3919,6 +3927,7 @@ cudaError_t launch_reduce1(bool pdl, const double* partials, int nparts, double*
 // for the extra plane of z halo); 0 if even whole columns need
 // more partial-sum slots than `cap` (blocks = column tiles x chunks x
 // members).
+template <int TY>
 int fx_planes(int n, int members, int64_t cap) {
   int dev = 0, sms = 0, occ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -3926,15 +3935,15 @@ int fx_planes(int n, int members, int64_t cap) {
       sms < 1)
     sms = 152;
   // resident blocks per SM: the waves are counted in units of sms * occ
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_defect64_fx, kFxTX * kFxTY,
-                                                    kFxSmem) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_defect64_fx<TY>, kFxTX * TY,
+                                                    kFxSmem<TY>) != cudaSuccess ||
       occ < 1) {
     cudaGetLastError();
     occ = 1;
   }
   const int64_t slots = (int64_t)sms * occ;
   const int64_t tiles =
-      (int64_t)((n + kFxTX - 1) / kFxTX) * ((n + kFxTY - 1) / kFxTY) * members;
+      (int64_t)((n + kFxTX - 1) / kFxTX) * ((n + TY - 1) / TY) * members;
   int best = 0;
   double best_cost = 0.0;
   for (int chunks = 1; chunks <= n; ++chunks) {
@@ -3951,6 +3960,15 @@ int fx_planes(int n, int members, int64_t cap) {
   return best;
 }
 
+// Whether blocks of TY rows and zc planes fit the partial-sum buffer and grid.
+template <int TY>
+bool fx_fits(int n, int members, int64_t cap, int zc) {
+  const int64_t chunks = (n + zc - 1) / zc;
+  const int64_t blocks =
+      (int64_t)((n + kFxTX - 1) / kFxTX) * ((n + TY - 1) / TY) * chunks * members;
+  return blocks <= cap && chunks * members <= 65535;
+}
+
 cudaError_t launch_defect64(const Lvl& L, const double* phi, const double* mu,
                             const double* om, const double* S1, const double* S2,
                             const double* S3, const double* b, float* r1, float* r2, float* r3,
@@ -3962,18 +3980,25 @@ cudaError_t launch_defect64(const Lvl& L, const double* phi, const double* mu,
   if (decided) *decided = false;
   if (!Mx) {
     const int64_t cap = (int64_t)kReduceBlocks * kReduceComps;
-    int zc = fx_planes(L.n, members, cap);
+    int ty = 4, zc = fx_planes<4>(L.n, members, cap);
+    if (zc == 0) {
+      ty = 8;
+      zc = fx_planes<8>(L.n, members, cap);
+    }
     if (planes > 0 && zc > 0) {
-      // a fixed choice, where its blocks fit the partial-sum buffer and grid
-      const int z = planes < L.n ? planes : L.n, ch = (L.n + z - 1) / z;
-      const int64_t blocks = (int64_t)((L.n + kFxTX - 1) / kFxTX) *
-                             ((L.n + kFxTY - 1) / kFxTY) * ch * members;
-      if (blocks <= cap && (int64_t)ch * members <= 65535) zc = z;
+      // a fixed choice, where its blocks fit
+      const int z = planes < L.n ? planes : L.n;
+      const bool four = fx_fits<4>(L.n, members, cap, z);
+      if (four || fx_fits<8>(L.n, members, cap, z)) {
+        ty = four ? 4 : 8;
+        zc = z;
+      }
     }
     if (zc > 0) {
       const int chunks = (L.n + zc - 1) / zc;
-      const dim3 grid((L.n + kFxTX - 1) / kFxTX, (L.n + kFxTY - 1) / kFxTY, chunks * members);
-      cudaError_t e = launch_ex(pdl, k_defect64_fx, grid, dim3(kFxTX * kFxTY), kFxSmem, st, L, zc, phi,
+      const dim3 grid((L.n + kFxTX - 1) / kFxTX, (L.n + ty - 1) / ty, chunks * members);
+      cudaError_t e = launch_ex(pdl, ty == 4 ? k_defect64_fx<4> : k_defect64_fx<8>, grid,
+                                dim3(kFxTX * ty), ty == 4 ? kFxSmem<4> : kFxSmem<8>, st, L, zc, phi,
                                 mu, om, S1, S2, S3, b, r1, r2, r3, q, partials, lap, c1m, lapmu,
                                 lapom);
       if (e == cudaSuccess)
