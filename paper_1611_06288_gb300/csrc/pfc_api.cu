@@ -990,8 +990,10 @@ int pfc_set_state(pfc_ctx* c, const double* any_phi, const double* any_phi_prev)
   const int64_t n3 = (int64_t)c->p.n * c->p.n * c->p.n * c->nb;
   const size_t bytes = (size_t)n3 * sizeof(double);
   PFC_CUDA(cudaMemcpyAsync(c->ring[c->ib], any_phi, bytes, cudaMemcpyDefault, c->st));
-  PFC_CUDA(cudaMemcpyAsync(c->ring[c->ic], any_phi_prev ? any_phi_prev : any_phi, bytes,
-                           cudaMemcpyDefault, c->st));
+  // without a previous state the Laplacian's pass copies the field
+  if (any_phi_prev || df_state(&c->p))
+    PFC_CUDA(cudaMemcpyAsync(c->ring[c->ic], any_phi_prev ? any_phi_prev : any_phi, bytes,
+                             cudaMemcpyDefault, c->st));
   if (df_state(&c->p)) {
     // PFC_MIXED_DF keeps phi as df pairs: convert in place
     PFC_CUDA(launch_df_from_f64(n3, c->ring[c->ib], as_df(c->ring[c->ib]), c->st));
@@ -1000,9 +1002,10 @@ int pfc_set_state(pfc_ctx* c, const double* any_phi, const double* any_phi_prev)
     PFC_CUDA(launch_laplacian_df(c->p.n, as_df(c->ring[c->ic]), as_df(c->lap[c->ic]), c->st));
     c->prof.launches += 4;
   } else {
-    PFC_CUDA(launch_laplacian(c->p.n, c->ring[c->ib], c->lap[c->ib], c->st, c->nb));
-    PFC_CUDA(launch_laplacian(c->p.n, c->ring[c->ic], c->lap[c->ic], c->st, c->nb));
-    c->prof.launches += 2;
+    PFC_CUDA(launch_state_laplacians(c->p.n, c->ring[c->ib], c->lap[c->ib],
+                                     any_phi_prev ? c->ring[c->ic] : nullptr, c->ring[c->ic],
+                                     c->lap[c->ic], c->st, c->nb));
+    c->prof.launches += 1;
   }
   if (variable_mobility(&c->p)) {
     // reference mobility of the FP32 correction solve: m0 + m2 mean(phi^2)

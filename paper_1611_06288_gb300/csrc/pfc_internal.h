@@ -185,9 +185,10 @@ cudaError_t launch_residual_norm2(const Lvl& L, const double* phi, const double*
 // decision to take (single member) it is part of the same launch (*decided).
 cudaError_t launch_reduce1(bool pdl, const double* partials, int nparts, double* out, int members,
                            cudaStream_t st, const DecideArgs* da, bool* decided);
-// Unscaled 7-point Laplacian (neighbour sum - 6 centre) of a field.
-cudaError_t launch_laplacian(int n, const double* v, double* lap, cudaStream_t st,
-                             int members = 1);
+// Unscaled 7-point Laplacians (neighbour sum - 6 centre) of a state's fields b and
+// c; c null: c is b, whose values go to copy.
+cudaError_t launch_state_laplacians(int n, const double* b, double* lapb, const double* c,
+                                    double* copy, double* lapc, cudaStream_t st, int members);
 // S2, S3 from b and the stored unscaled Laplacians of b and c.
 cudaError_t launch_source_cached(const Lvl& L, const double* b, const double* lapb,
                                  const double* lapc, double* S2, double* S3, cudaStream_t st,

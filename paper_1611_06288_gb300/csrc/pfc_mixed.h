@@ -143,7 +143,7 @@ cudaError_t launch_diagnostics_df(int n, const float2* a, const float2* b, doubl
 cudaError_t launch_round_f32(int64_t count, const double* x, float* y, cudaStream_t st);
 cudaError_t launch_widen_f64(int64_t count, const float* x, double* y, cudaStream_t st);
 
-// df counterparts of launch_laplacian, launch_source_cached and
+// df counterparts of launch_state_laplacians (one field), launch_source_cached and
 // launch_diagnostics_cached.
 cudaError_t launch_laplacian_df(int n, const float2* v, float2* lap, cudaStream_t st);
 cudaError_t launch_source_cached_df(const Lvl& L, const float2* b, const float2* lapb,
