@@ -77,10 +77,10 @@ START_BYTES = {"previous": 104.0, "extrapolate_all": 176.0}
 # DRAM bytes (read + write) of one launch of a kernel class of a precision,
 # from the ncu capture summarised in profiles/ (cold L2); absent where no
 # capture of the current kernel exists.
-# The defect class of the mixed path is the full defect (150.8 MB a launch);
+# The defect class of the mixed path is the full defect (149.9 MB a launch);
 # the start of a step has a class of its own.  Keyed by the finest level's
 # size the capture ran at (other sizes: null).
-NCU_TRAFFIC = {("mixed", "defect", 128): 150.8e6,   # profiles/k_defect64_fx_128.md
+NCU_TRAFFIC = {("mixed", "defect", 128): 149.9e6,   # profiles/k_defect64_fx_128.md
                # the start from the three-field extrapolation:
                ("mixed", "start", 128, "extrapolate_all"): 319.0e6}  # k_start64_extrap_128.md
 

@@ -133,8 +133,8 @@ typedef struct pfc_params {
                                 state changes; 0 (default): they are formed
                                 on request */
   int    defect_planes;      /* PFC_MIXED: planes per thread block of the FP64
-                                defect (its tiles are 32 x 8 cells x this many
-                                planes); 0 (default) chooses them from the SM
+                                defect (its tiles are 32 x 4 cells, or 32 x 8 in
+                                large ensembles, x this many planes); 0 (default) chooses them from the SM
                                 count (fewest waves), a value > 0 fixes them
                                 (an autotuner's choice; larger than n means
                                 n) */
