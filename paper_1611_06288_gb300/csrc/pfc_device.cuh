@@ -215,15 +215,21 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-// a / d for d >= 1 in 5 FP64 operations (a division is about 10, and the FP64
-// pipe is what bounds the smoother): the FP32 reciprocal of d, one Newton step
-// r (2 - d r) to about 2^-46, and the quotient a r corrected by its exact
-// remainder a - d q, which leaves the rounding of the last operation.  Beyond
-// FP32's range (or NaN) the division itself.
+// a / d in 5 FP64 operations (a division is about 10, and the FP64 pipe is what
+// bounds the smoother): Newton's iteration for the reciprocal and a quotient
+// corrected by its remainder (P. Markstein, Computation of elementary functions
+// on the IBM RISC System/6000 processor, IBM J. Res. Dev. 34, 1990).  The FP32
+// reciprocal of d rounded to FP32 is right to 2^-23 + 2^-24 < 2^-22.4, one Newton
+// step r (2 - d r) makes that 2^-44.8, and q = a r plus r times its remainder
+// a - d q is right to 2^-89 before the last operation rounds it.  Where the FP32
+// reciprocal is not normal (d outside [1, 2^123)) or d q may not be finite
+// (|a| >= 2^1022, infinities, NaN) the division itself; both tests read exponents
+// on the integer pipe.
 __device__ __forceinline__ double div_by(double a, double d) {
-  const float df = d2f_rn(d);
-  if (!(df < 1e37f)) return a / d;
-  double r = f2d(rcp_approx(df));
+  const unsigned ha = (unsigned)__double2hiint(a) & 0x7FFFFFFFu;
+  const unsigned hd = (unsigned)__double2hiint(d);
+  if (ha >= (2045u << 20) || hd - (1023u << 20) >= (123u << 20)) return a / d;
+  double r = f2d(rcp_approx(d2f_rn(d)));
   r = fma(r, fma(-d, r, 1.0), r);
   const double q = a * r;
   return fma(r, fma(-d, q, a), q);
