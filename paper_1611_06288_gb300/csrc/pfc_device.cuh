@@ -206,9 +206,9 @@ __device__ __forceinline__ double f2d(float f) {
   return __hiloint2double((int)hi, (int)(u << 29));
 }
 
-// 1/x within 1 ulp for a normal x, without the scaling of subnormal divisors
-// that __fdividef carries: num * rcp_approx(det) equals __fdividef(num, det)
-// for the determinants of the pointwise solve, which are >= 1.
+// 1/x by PTX's rcp.approx.ftz.f32, whose documented error is at most one ulp
+// (subnormal divisors count as zero, subnormal results become zero).  A quotient
+// num * rcp_approx(det) is then within 2^-23 + 2^-24 of num / det, relative.
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

@@ -1177,7 +1177,7 @@ __device__ __forceinline__ void lin_point(const LvlF& L, float sp, float sm_, fl
   const float st3 = fmaf(L.gh, sp, r3);
   const float Q = q + L.Q0;
   const float det = fmaf(L.kap, Q, 1.0f);
-  // the division by the 2x2 determinant within 2 ulp: an FP32 preconditioner
+  // the quotient by the determinant to 2^-22.4 (rcp_approx): an FP32 preconditioner
   // step, and the IEEE division was a fifth of the sweep's instructions
   dm = fmaf(Q, st1, fmaf(-L.g6, st3, st2)) * rcp_approx(det);
   dp = fmaf(-L.kap, dm, st1);

@@ -89,3 +89,29 @@ def test_quotient_by_negative_determinants(j):
     ref = S2[colour0()] / det
     got = first_mu(B.PFC_NEWTON, e, S2, np.zeros((N, N, N)), 1.0 + 2.0 ** j)
     assert (np.abs(got - ref) <= np.spacing(np.abs(ref))).all()
+
+
+# n = 6: one cell a thread; 16: two
+@pytest.mark.parametrize("n", [6, 16])
+@pytest.mark.parametrize("e", [-4, 0, 3, 10, 19])
+def test_fp32_quotient_within_its_bound(n, e):
+    """The FP32 solve's quotient: a reciprocal to one ulp, 2^-23 relative, and one
+    rounded product, 2^-24.  One Jacobi sweep of weight 1 from zero with r1 = r3 = 0
+    leaves d2 = r2 times it; det from just above 1 to 2^121."""
+    rng = np.random.default_rng(n + e)
+    f32 = lambda x: np.asarray(x).astype(np.float32)
+    Q0, kap = 18.0 * 2.0 ** (4 * e), 6.0 * 2.0 ** (2 * e)
+    q = f32(Q0 * 10.0 ** rng.uniform(-3, 0.5, n ** 3))
+    r2 = f32(rng.choice([-1.0, 1.0], n ** 3) * np.ldexp(rng.uniform(1, 2, n ** 3),
+                                                        rng.integers(0, 41, n ** 3)))
+    # kap Q + 1 rounded once: kap Q is exact here, and a 1 below its last place still
+    # ends a tie
+    kq = kap * f32(q.astype(float) + Q0).astype(float)
+    det = f32(np.where(kq + 1.0 == kq, np.nextafter(kq, np.inf), kq + 1.0)).astype(float)
+    z = lambda: torch.zeros(n ** 3, device="cuda")
+    d, t = [z() for _ in range(3)], [z() for _ in range(3)]
+    up = lambda x: dev(x, torch.float32)
+    B.pfc_op_lin_jacobi(n, 2.0 ** -e, 0.0, 1.0, 1, 1.0, True, *d, *t, z(), up(r2), z(), up(q))
+    ref = r2.astype(float) / det
+    bound = (2.0 ** -23 + 2.0 ** -24) * (1 + 2.0 ** -23)
+    assert (np.abs(host(d[1]) - ref) <= bound * np.abs(ref)).all()
