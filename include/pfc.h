@@ -114,17 +114,14 @@ typedef struct pfc_params {
                                 thread-block cluster per member (levels in z
                                 slabs over the CTAs, neighbour planes through
                                 distributed shared memory) where the device
-                                can run such a cluster; 2 uses the cluster
-                                only for levels of at most 16^3 cells, and
-                                there only where they do not fit the
-                                single-block tail, which takes less time
-                                (348 against 352 us a step on the 128^3
-                                smooth-mode workload), the levels above
-                                keeping their full-GPU launches; 0 (default)
-                                keeps separate launches down to 16^3 and one
-                                block below, faster for ensembles.  Same
-                                arithmetic up to summation order and the
-                                approximate division of the pointwise solve */
+                                can run such a cluster; 0 (default) keeps
+                                separate launches down to 16^3 and one block
+                                below, faster for ensembles.  2 is accepted
+                                and means 0: one block takes the levels of at
+                                most 16^3 cells in less time than a cluster
+                                (128^3 smooth-mode workload 348 against 352 us
+                                a step).  Same arithmetic up to summation
+                                order */
   int    step_diagnostics;   /* 1: every step also forms the energy/mass sums
                                 of its new state in the same graph launch
                                 (no further launch or synchronisation), and

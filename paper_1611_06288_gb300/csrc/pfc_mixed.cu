@@ -2891,6 +2891,10 @@ int tail_threads(int n) {
 }
 
 constexpr size_t kTailMaxSmem = 200 * 1024;   // + static shared memory <= 227 KiB
+static_assert(kTailMaxN == 16 && kTailMaxLevels >= 4 &&
+                  (tail_floats(16) + tail_floats(8) + tail_floats(4) + tail_floats(2)) *
+                          sizeof(float) <= kTailMaxSmem,
+              "the longest chain of levels fits one block");
 
 // ---------------------------------------------------------------------------
 // Cluster tail: the coarse part of an FP32 V-cycle from a level of up to
@@ -3773,13 +3777,8 @@ cudaError_t ctail32(const Ctx32& c, int l0, bool zero_init, int nd, size_t smem,
 }
 
 // Whether the single-block tail takes the levels from l on (where the cluster
-// tail does not).
-bool block_tail_at(const Ctx32& c, int l) {
-  if (c.L[l].n > kTailMaxN || c.nl - l > kTailMaxLevels) return false;
-  int sizes[kMaxLevelsMixed];
-  for (int q = 0; q < c.nl; ++q) sizes[q] = c.L[q].n;
-  return tail_smem_bytes(sizes, l, c.nl) <= kTailMaxSmem;
-}
+// tail does not): every level chain from kTailMaxN^3 cells down fits one block.
+bool block_tail_at(const Ctx32& c, int l) { return c.L[l].n <= kTailMaxN; }
 
 // rho = r - J d (r where zero: d = 0) averaged onto the next level.
 cudaError_t launch_lin_restrict(bool pdl, const LvlF& L, bool zero, int members, const float* d1,
@@ -3825,12 +3824,8 @@ int chain_extra(const Ctx32& c, int l) {
 cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
   MixedBufs& mx = *c.mx;
   const LvlF& L = c.L[l];
-  // cluster tail: from the first level of at most kCtMaxN^3 cells (mode 1), or
-  // (mode 2) only on levels of the single-block tail that do not fit one
-  // block: where both can run, one block takes less time (the 128^3 smooth run
-  // 348 against 352 us a step, 64^3 alike)
-  if (c.p->cluster_tail == 1 ||
-      (c.p->cluster_tail == 2 && L.n <= kTailMaxN && !block_tail_at(c, l))) {
+  // cluster tail: from the first level of at most kCtMaxN^3 cells
+  if (c.p->cluster_tail == 1) {
     size_t smem = 0;
     int ga_off = 0;
     const int nd = ctail_layout(c, l, &smem, &ga_off);

@@ -26,7 +26,7 @@ struct TLev {
   int hc, cs;                            // cells of a colour, distance of the colours
 };
 
-__host__ __device__ inline int tail_floats(int n) { return 10 * (n * n * n + 32); }
+__host__ __device__ constexpr int tail_floats(int n) { return 10 * (n * n * n + 32); }
 
 __device__ __forceinline__ TLev tlev(const TailParams& P, int l) {
   const int n = P.L[l].n;

@@ -171,8 +171,8 @@ def smooth_sweep(n: int, dt: float = 0.0125, tol: float = 1e-9):
     Mixed-path settings: at n >= 64 the finest level is stiff (red-black) and
     V(0,1) cycles are fastest, two per correction with 4 Jacobi sweeps per
     requested sweep on the intermediate levels; at 32^3 V(1,2).  Below 256^3
-    cluster_tail is 2 (the coarsest levels on a cluster only where one block
-    does not hold them).
+    cluster_tail is 2, which the library takes as 0 (one block for the levels
+    of at most 16^3 cells).
 
     Timed runs start each step from u^{k+1} := 2 u^k - u^{k-1} in phi, mu and
     omega (guess extrapolate_all): the first defect falls from 2.3e-5 to
