@@ -2404,98 +2404,13 @@ __global__ void __launch_bounds__(kPsTX * TY) k_lin_prolong_sweep32(
   }
 }
 
-// Coarsest level of the linear problem when it is not part of a tail launch:
-// start from zero, sweeps in one block (red-black, kind 0, or damped Jacobi
-// through t, kind 1) until the largest change is below 1e-6 of the largest
-// value or max_sweeps.  Split layout.
-__global__ void k_lin_coarse_solve32(LvlF L, int kind, float w, int max_sweeps, float* d1,
-                                     float* d2, float* d3, float* t1, float* t2, float* t3,
-                                     const float* r1, const float* r2, const float* r3,
-                                     const float* q) {
-  __shared__ float red[2][32];
-  __shared__ int done;
-  const int n = L.n, half = n >> 1;
-  const int cells = n * n * n, ccells = half * n * n;
-  const size_t off = (size_t)blockIdx.x * cells;     // one block per member
-  d1 += off, d2 += off, d3 += off, t1 += off, t2 += off, t3 += off;
-  r1 += off, r2 += off, r3 += off, q += off;
-  for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-    d1[t] = 0.f;
-    d2[t] = 0.f;
-    d3[t] = 0.f;
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    float change = 0.f, size = 0.f;
-    if (kind == PFC_SWEEP_JACOBI) {
-      for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-        int p, j, k, colour;
-        split_cell(t, n, p, j, k, colour);
-        const Stencil s = split_stencil(p, j, k, colour, n);
-        float dp, dm, dw;
-        lin_point(L, nbsum_coherent(d1, s), nbsum_coherent(d2, s), nbsum_coherent(d3, s),
-                  q[s.c], r1[s.c], r2[s.c], r3[s.c], dp, dm, dw);
-        t1[s.c] = fmaf(w, dp - d1[s.c], d1[s.c]);
-        t2[s.c] = fmaf(w, dm - d2[s.c], d2[s.c]);
-        t3[s.c] = fmaf(w, dw - d3[s.c], d3[s.c]);
-      }
-      __syncthreads();
-      for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-        change = fmaxf(change, fmaxf(fabsf(t1[t] - d1[t]),
-                                     fmaxf(fabsf(t2[t] - d2[t]), fabsf(t3[t] - d3[t]))));
-        size = fmaxf(size, fmaxf(fabsf(t1[t]), fmaxf(fabsf(t2[t]), fabsf(t3[t]))));
-        d1[t] = t1[t];
-        d2[t] = t2[t];
-        d3[t] = t3[t];
-      }
-      __syncthreads();
-    } else {
-      for (int colour = 0; colour < 2; ++colour) {
-        for (int t = threadIdx.x; t < ccells; t += blockDim.x) {
-          const int p = t % half, rr = t / half;
-          const Stencil s = split_stencil(p, rr % n, rr / n, colour, n);
-          float dp, dm, dw;
-          lin_point(L, nbsum_coherent(d1, s), nbsum_coherent(d2, s), nbsum_coherent(d3, s),
-                    q[s.c], r1[s.c], r2[s.c], r3[s.c], dp, dm, dw);
-          change = fmaxf(change, fmaxf(fabsf(dp - d1[s.c]),
-                                       fmaxf(fabsf(dm - d2[s.c]), fabsf(dw - d3[s.c]))));
-          size = fmaxf(size, fmaxf(fabsf(dp), fmaxf(fabsf(dm), fabsf(dw))));
-          d1[s.c] = dp;
-          d2[s.c] = dm;
-          d3[s.c] = dw;
-        }
-        __syncthreads();
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      change = fmaxf(change, __shfl_down_sync(0xffffffffu, change, o));
-      size = fmaxf(size, __shfl_down_sync(0xffffffffu, size, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      red[0][threadIdx.x >> 5] = change;
-      red[1][threadIdx.x >> 5] = size;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float c = 0.f, z = 0.f;
-      for (int v = 0; v < (int)((blockDim.x + 31) >> 5); ++v) {
-        c = fmaxf(c, red[0][v]);
-        z = fmaxf(z, red[1][v]);
-      }
-      done = (c <= 1e-6f * z);
-    }
-    __syncthreads();
-    if (done) break;
-  }
-}
-
 // ---------------------------------------------------------------------------
-// Coarse tail: every level of at most kTailMaxN^3 cells of one FP32 V-cycle
-// (pre-smoothing, residual + restriction, coarsest solve, prolongation +
-// correction, post-smoothing) in a single launch of one thread block whose
-// levels all live in shared memory.  On these grids separate kernels were
-// pure launch latency.  Each thread owns a fixed (i, j) column and walks k
-// with a stride, so no cell index is divided per cell.
+// Coarse levels of one FP32 V-cycle (pre-smoothing, residual + restriction,
+// coarsest solve, prolongation + correction, post-smoothing) in a single launch:
+// on these grids separate kernels were pure launch latency.  Every level of at
+// most kTailMaxN^3 cells goes to one block with the levels in shared memory
+// (pfc_tail.cuh); or, as an option, levels of up to kCtMaxN^3 cells to a
+// thread-block cluster (below).
 // ---------------------------------------------------------------------------
 constexpr int kTailMaxN = 16;
 constexpr int kTailMaxLevels = 8;
@@ -2515,7 +2430,12 @@ struct TailParams {
   const float* gq;
 };
 
-// Fields of one level in shared memory: d(3), t(3), r(3), q, n^3 floats each.
+// The levels below the cluster's, which its CTA 0 holds in shared memory in natural
+// order: each thread owns a fixed (i, j) column and walks k with a stride, so no
+// cell index is divided per cell.  (The one-block tail orders them by colour,
+// pfc_tail.cuh.)
+//
+// Fields of one level: d(3), t(3), r(3), q, n^3 floats each.
 struct SLev {
   float *d0, *d1, *d2, *t0, *t1, *t2, *r0, *r1, *r2, *q;
 };
@@ -2827,25 +2747,7 @@ __device__ void tail_coarse(const LvlF& L, int kind, SLev S, float w, int max_sw
   }
 }
 
-// q of every tail level below the first, restricted in shared memory.
-__device__ void tail_qrestrict(float* smem, const TailParams& P) {
-  for (int l = 1; l < P.nlev; ++l) {
-    const SLev F = slev(smem, P, l - 1), C = slev(smem, P, l);
-    const int n = P.L[l - 1].n;
-    const Walk W(n >> 1);
-    if (W.active) {
-      for (int K = W.k0; K < W.n; K += W.kstep) {
-        float acc = 0.f;
-        for (int ch = 0; ch < 8; ++ch)
-          acc += F.q[(2 * W.i + (ch & 1)) + n * ((2 * W.j + ((ch >> 1) & 1)) + n * (2 * K + (ch >> 2)))];
-        C.q[W.i + W.n * (W.j + W.n * K)] = 0.125f * acc;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// One V-cycle over the tail levels held in shared memory (one block).
+// One V-cycle over CTA 0's levels.
 __device__ void tail_vcycle(float* smem, const TailParams& P, bool zero_top, float (*red)[32],
                             int* done) {
   const int last = P.nlev - 1;
@@ -3798,7 +3700,7 @@ cudaError_t launch_lin_restrict(bool pdl, const LvlF& L, bool zero, int members,
 }
 
 // Whether vcycle32 at level l restricts to l + 1 with a launch of its own
-// (not the cluster tail, the shared-memory tail or the coarsest solve).
+// (not the cluster tail or the shared-memory tail).
 bool restricts_alone(const Ctx32& c, int l) {
   return c.p->cluster_tail != 1 && l < c.nl - 1 && !block_tail_at(c, l);
 }
@@ -3831,18 +3733,9 @@ cudaError_t vcycle32(const Ctx32& c, int l, bool zero_init, int have = 0) {
     const int nd = ctail_layout(c, l, &smem, &ga_off);
     if (nd > 0 && ctail_supported()) return ctail32(c, l, zero_init, nd, smem, ga_off);
   }
+  // the coarsest level, of at most 16^3 cells (validate), always goes there
   if (block_tail_at(c, l)) return tail32(c, l, zero_init);
-  if (l == c.nl - 1) {
-    const int work = L.n * L.n * L.n;
-    int threads = ((work + 31) / 32) * 32;
-    if (threads > 1024) threads = 1024;
-    prof_begin(c.pr, PFC_K_LIN_COARSE, c.st);
-    k_lin_coarse_solve32<<<c.nb, threads, 0, c.st>>>(
-        L, c.kind[l], c.w, 400, mx.d[l][0], mx.d[l][1], mx.d[l][2], mx.t[l][0], mx.t[l][1],
-        mx.t[l][2], mx.r[l][0], mx.r[l][1], mx.r[l][2], mx.q[l]);
-    prof_end(c.pr, PFC_K_LIN_COARSE, l, 1, c.st);
-    return cudaGetLastError();
-  }
+  if (l == c.nl - 1) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
   // without pre-smoothing from a zero start d stays 0 until the prolongation,
   // which then assigns instead of adding
