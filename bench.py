@@ -50,7 +50,7 @@ KERNEL_BYTES = {
     "smooth": (40.0, 1),          # per colour pass: half of (u 24 + S2,S3 16 + b 8 + phi 8 + write u 24)
     "residual_norm": (56.0, 2),   # read u, b, S2, S3 (48), write the Laplacian of phi (8)
     "residual_restrict": (57.0, 1),
-    "prolong": (57.0, 2),
+    "prolong": (54.0, 1),         # read+write u (48), coarse v and w (48/8)
     "source": (32.0, 1),
     "restrict": (9.0, 1),
     "coarse_source": (80.0, 1),
@@ -238,7 +238,7 @@ class ClockSampler:
 # restriction reads only r (12 + 12/8) and the prolongation assigns d
 # (12 + 12/8).  A red-black sweep is two colour passes of 20 B/cell (half
 # of: d 12, r and q 16, d written 12); a damped Jacobi sweep reads d, r, q
-# and writes t (40 B/cell), an odd count adds one copy back (24 B/cell).
+# and writes t (40 B/cell; after an odd count d and t change places).
 # The coarse tail (from the first level of at most 16^3 cells) reads r and q
 # and writes d of its top level (28 B/cell); its lower levels stay in
 # shared memory.
@@ -285,10 +285,11 @@ def vcycle_bytes(params, levels):
         total += cells * (dbytes + 1.5)
         if kind == B.PFC_SWEEP_JACOBI:
             sweeps = params.nu2 * (params.jacobi_factor0 if first else params.jacobi_factor)
-            total += cells * (40.0 * sweeps + (24.0 if sweeps % 2 else 0.0))
-            if sweeps > 0 and m % 32 == 0:
-                # the prolongation fused into the first sweep: d + P e stays
-                # in shared memory (not written, not read back)
+            total += cells * 40.0 * sweeps
+            if sweeps > 0 and m % 32 == 0 and m ** 3 <= 1 << 20:
+                # the prolongation fused into the first sweep, on levels where
+                # that pays: d + P e stays in shared memory (not written, not
+                # read back)
                 total -= cells * 24.0
         else:
             total += cells * 40.0 * params.nu2
@@ -431,10 +432,11 @@ def run_reference(args):
 # ---------------------------------------------------------------------------
 
 # FP64 FAS smoother: FP64 flops per updated cell of one launch (a red-black
-# colour pass updates n^3/2 cells, a Jacobi sweep n^3): three neighbour sums
-# (15 DADD), the source terms, the Newton coefficient and its cubic, and the
-# 3x3 solve by elimination with one division (k_smooth_colour, Section 5).
-FP64_SMOOTH_FLOPS = 66.0
+# colour pass updates n^3/2 cells, a Jacobi sweep n^3, whose damping's 9 flops are
+# not counted): three neighbour sums (15 DADD) and the pointwise Newton solve, 17
+# DFMA + 1 DADD + 5 DMUL with its quotient (k_smooth_colour, Section 5; ncu counts
+# the same, profiles/k_smooth_colour_128.md).
+FP64_SMOOTH_FLOPS = 55.0
 
 
 def fp64_class_roofline(cls, m, red_black, launches, ms, hbm_gbs, hbm_source):
