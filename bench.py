@@ -42,7 +42,8 @@ WORKLOAD = {"workload": "smooth-mode 128^3", "n": 128, "L": 32.0, "eps": 0.025,
 # Algorithmic bytes per cell of one counted launch, and launches per timed
 # group, for each kernel class (minimum traffic: every field touched once).
 KERNEL_BYTES = {
-    "defect": (64.0, 2),          # read df phi,mu,om,b,S2,S3 (48) write r32 x3, q32 (16)
+    "defect": (72.0, 2),          # read df phi,mu,om,b,S2,S3 (48) write r32 x3, q32 (16) and the
+                                  # Laplacian of phi (8)
     "lin_smooth": (20.0, 1),      # per colour pass: half of read d (12) + r,q (16) + write d (12)
     "lin_restrict": (29.5, 1),    # read d,r,q (28) + write coarse r (12/8)
     "lin_prolong": (25.5, 1),     # read+write d (24) + coarse d (12/8)

@@ -7,8 +7,9 @@
 // Two sweeps, us, two launches of k_lin_jacobi32m / one of this: 256^3 204 /
 // 161, 192^3 99 / 68, 160^3 61 / 43, 132^3 33 / 30, 6 x 128^3 158 / 117, 3 x
 // 96^3 36 / 28, 8 x 80^3 59 / 49, 42 x 64^3 139 / 110, 39 x 48^3 61.6 / 53.8, 60
-// x 40^3 60 / 49.  What bounds it: the L1 / shared-memory pipe (140 wavefronts a
-// warp and plane), and the latency that 16 warps an SM leave.
+// x 40^3 60 / 49.  What bounds it: the latency that 16 warps an SM (126 registers a
+// thread) leave; no unit is full at 256^3 (ncu: issue 48 %, L1 / shared-memory pipe
+// 47 % with 128 wavefronts a warp and plane, DRAM 53 %).
 //
 // A block owns whole rows (so that a row's neighbours are in the block, every
 // access of a warp is aligned, and a plane of the tile is one range of memory)

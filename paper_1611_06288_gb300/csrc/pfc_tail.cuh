@@ -10,9 +10,9 @@
 // were bank conflicts), a thread's positions and their neighbours are the same
 // indices for both colours and are worked out once per call, and r, q of a
 // thread's cells stay in registers over the sweeps of a call.  Measured (ncu):
-// V(2,2) on 16^3 with four coarsest sweeps on 8^3 36.4 -> 19.6 us (a colour pass
-// of 16^3 takes 0.85 us, 0.65 at the shared-memory rate), 16^3 alone with two
-// sweeps 16.4 -> 8.3.
+// V(2,2) on 16^3 with four coarsest sweeps on 8^3 36.4 -> 19.6 us, 9.2 of them at
+// the shared-memory rate (19.1 k wavefronts), the SM issuing 57 % of the time; 16^3
+// alone with two sweeps 16.4 -> 9.6 (warm caches).
 
 extern __shared__ float tsm[];
 
